@@ -128,33 +128,45 @@ def _activations(gen, rows, n, vision):
     return x.to(torch.bfloat16)
 
 
-def _transform(case, n, seed):
-    t = synth.make_transform(n, seed, case["geometry"], clip=case["clip"], gr=case["gr"], gc=case["gc"])
+def _factors(case, n, seed):
+    return synth.make_transform(n, seed, case["geometry"], clip=case["clip"], gr=case["gr"], gc=case["gc"])
+
+
+def _transform(case, n, t):
     return B.batq_transform_create(n, t.left, t.right, t.clip_lo, t.clip_hi, gr=case["gr"], gc=case["gc"])
 
 
-def prepare(case, seed):
+def _inputs(case, seed):
+    """(factors, weight or None, activations) of every call of a pass, in order."""
     gen = torch.Generator(device="cuda")
     gen.manual_seed(seed)
     if case["kind"] == "quantise":
+        yield _factors(case, case["n"], seed), None, _activations(gen, case["rows"], case["n"], 0.0)
+        return
+    for i, (n, m) in enumerate(_projections(case)):
+        weight = (torch.randn((m, n), generator=gen, device="cuda") * 0.02).to(torch.bfloat16)
+        yield _factors(case, n, seed * 64 + i), weight, _activations(gen, case["tokens"], n, case.get("vision", 0.0))
+
+
+def prepare(case, seed):
+    if case["kind"] == "quantise":
         rows, n = case["rows"], case["n"]
+        (t, _, x), = _inputs(case, seed)
         fp8 = case["format"] == "mxfp8"
         layout = B.SF_MMA if case["layout"] == "mma" else B.SF_ROWMAJOR
         return {"run": _run_quantise, "fn": B.batq_quantize_act_mxfp8 if fp8 else B.batq_quantize_act,
-                "t": _transform(case, n, seed), "x": _activations(gen, rows, n, 0.0), "layout": layout,
+                "t": _transform(case, n, t), "x": x, "layout": layout,
                 "codes": torch.zeros((rows, n if fp8 else n // 2), dtype=torch.uint8, device="cuda"),
                 "scales": torch.zeros(B.batq_sf_bytes(rows, n, layout), dtype=torch.uint8, device="cuda")}
     tokens, a8 = case["tokens"], case["format"] == "w4a8"
     out = torch.float32 if case.get("out") == "f32" else torch.bfloat16
     calls, need = [], 0
-    for i, (n, m) in enumerate(_projections(case)):
-        t = _transform(case, n, seed * 64 + i)
-        weight = (torch.randn((m, n), generator=gen, device="cuda") * 0.02).to(torch.bfloat16)
+    for (n, m), (t, weight, x) in zip(_projections(case), _inputs(case, seed)):
+        t = _transform(case, n, t)
         w = B.batq_prepare_weight(t, weight)
-        del weight
         need = max(need, B.batq_linear_w4a8_workspace_bytes(w, tokens) if a8 else B.batq_linear_workspace_bytes(w, tokens))
-        calls.append((t, w, _activations(gen, tokens, n, case.get("vision", 0.0)),
-                      torch.zeros((tokens, m), dtype=out, device="cuda")))
+        calls.append((t, w, x, torch.zeros((tokens, m), dtype=out, device="cuda")))
+    del weight
     state = {"run": _run_calls, "fn": B.batq_linear_w4a8 if a8 else B.batq_linear_w4a4, "calls": calls,
              "workspace": B.aligned_workspace(need), "out": [c[3] for c in calls]}
     if case.get("graph"):
@@ -209,3 +221,42 @@ def tolerance(case):
     if case["kind"] == "quantise":
         return {"rel": 5e-4, "differ": 2e-6}
     return {"rel": 4e-3}
+
+
+def _block_transform(v, left, right):
+    """vec(L^T V R) of every 32-element block of the rows of v, 64 bits."""
+    k, gr, gc = v.shape[1] // 32, left.shape[-1], right.shape[-1]
+    v = v.view(-1, k, gr, gc)
+    v = torch.matmul(v, right)                        # [rows, k, gr, gc] x [1 or k, gc, gc]
+    return torch.matmul(left.transpose(-1, -2), v).reshape(-1, k, 32)
+
+
+def _mx(v, emax):
+    """The values that MXFP4 (emax 2) or MXFP8 E4M3 (emax 8) keeps of blocks v [rows, k, 32]: shared scale
+    2^(floor(log2 amax) - emax), elements to the nearest, ties to even, saturating."""
+    e = (torch.frexp(v.abs().amax(-1, keepdim=True))[1] - 1 - emax).clamp(-127, 127)
+    u = torch.ldexp(v, -e)
+    low, bits, top = (0, 1, 6.0) if emax == 2 else (-6, 3, 448.0)   # exponent of the subnormals, mantissa bits, maximum
+    step = (torch.frexp(u)[1] - 1).clamp_min(low) - bits
+    u = torch.ldexp(torch.round(torch.ldexp(u, -step)), step).clamp(-top, top)
+    return torch.ldexp(u, e).reshape(v.shape[0], -1)
+
+
+def exact(case, seed):
+    """The results in 64 bits; nothing for codes and scale bytes, which are whole numbers."""
+    if case["kind"] == "quantise":
+        return None
+    emax, out = 8 if case["format"] == "w4a8" else 2, []
+    for t, weight, x in _inputs(case, seed):
+        left, right = (torch.from_numpy(f).cuda().double() for f in (t.left, t.right))
+        inverse_left, inverse_right = (torch.linalg.inv(f).transpose(-1, -2) for f in (left, right))
+        w = torch.cat([_mx(_block_transform(p.double(), inverse_left, inverse_right), 2) for p in weight.split(2048)])
+        y = []
+        for p in x.split(2048):
+            v = _block_transform(p.double(), left, right)
+            if t.clip_lo is not None:
+                lo, hi = (torch.from_numpy(c).cuda().double()[:, None] for c in (t.clip_lo, t.clip_hi))
+                v = torch.minimum(torch.maximum(v, lo * v.amin(-1, keepdim=True)), hi * v.amax(-1, keepdim=True))
+            y.append(_mx(v, emax) @ w.T)
+        out.append(torch.cat(y))
+    return out
