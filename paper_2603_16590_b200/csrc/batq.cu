@@ -166,14 +166,22 @@ batq_status device_setup(int* device_out, const DeviceInfo** info_out) {
     e = e ? e : set_smem(linear_small_s_fused_kernel<true, 4>, FusedCfg::kSmemBytes);
     e = e ? e : set_smem(linear_small_s_fused_kernel<false, 2>, FusedCfg::kSmemBytes);
     e = e ? e : set_smem(linear_small_s_fused_kernel<true, 2>, FusedCfg::kSmemBytes);
-    e = e ? e : set_smem(gemm_small_s_kernel<16, false>, SmallCfg<16>::kSmemBytes);
-    e = e ? e : set_smem(gemm_small_s_kernel<16, true>, SmallCfg<16>::kSmemBytes);
-    e = e ? e : set_smem(gemm_small_s_kernel<32, false>, SmallCfg<32>::kSmemBytes);
-    e = e ? e : set_smem(gemm_small_s_kernel<32, true>, SmallCfg<32>::kSmemBytes);
-    e = e ? e : set_smem(gemm_small_s_kernel<64, false>, SmallCfg<64>::kSmemBytes);
-    e = e ? e : set_smem(gemm_small_s_kernel<64, true>, SmallCfg<64>::kSmemBytes);
-    e = e ? e : set_smem(gemm_small_s_kernel<128, false>, SmallCfg<128>::kSmemBytes);
-    e = e ? e : set_smem(gemm_small_s_kernel<128, true>, SmallCfg<128>::kSmemBytes);
+    e = e ? e : set_smem(gemm_small_s_kernel<16, false, false>, SmallCfg<16, false>::kSmemBytes);
+    e = e ? e : set_smem(gemm_small_s_kernel<16, true, false>, SmallCfg<16, false>::kSmemBytes);
+    e = e ? e : set_smem(gemm_small_s_kernel<32, false, false>, SmallCfg<32, false>::kSmemBytes);
+    e = e ? e : set_smem(gemm_small_s_kernel<32, true, false>, SmallCfg<32, false>::kSmemBytes);
+    e = e ? e : set_smem(gemm_small_s_kernel<64, false, false>, SmallCfg<64, false>::kSmemBytes);
+    e = e ? e : set_smem(gemm_small_s_kernel<64, true, false>, SmallCfg<64, false>::kSmemBytes);
+    e = e ? e : set_smem(gemm_small_s_kernel<128, false, false>, SmallCfg<128, false>::kSmemBytes);
+    e = e ? e : set_smem(gemm_small_s_kernel<128, true, false>, SmallCfg<128, false>::kSmemBytes);
+    e = e ? e : set_smem(gemm_small_s_kernel<16, false, true>, SmallCfg<16, true>::kSmemBytes);
+    e = e ? e : set_smem(gemm_small_s_kernel<16, true, true>, SmallCfg<16, true>::kSmemBytes);
+    e = e ? e : set_smem(gemm_small_s_kernel<32, false, true>, SmallCfg<32, true>::kSmemBytes);
+    e = e ? e : set_smem(gemm_small_s_kernel<32, true, true>, SmallCfg<32, true>::kSmemBytes);
+    e = e ? e : set_smem(gemm_small_s_kernel<64, false, true>, SmallCfg<64, true>::kSmemBytes);
+    e = e ? e : set_smem(gemm_small_s_kernel<64, true, true>, SmallCfg<64, true>::kSmemBytes);
+    e = e ? e : set_smem(gemm_small_s_kernel<128, false, true>, SmallCfg<128, true>::kSmemBytes);
+    e = e ? e : set_smem(gemm_small_s_kernel<128, true, true>, SmallCfg<128, true>::kSmemBytes);
     if (e != cudaSuccess) { cudaGetLastError(); return BATQ_ERR_CUDA; }
     if (g_encode_tiled == nullptr) {
       void* fn = nullptr;
@@ -380,6 +388,69 @@ bool alu_small_geometry(const batq_transform* t) {
   return t == nullptr || t->gc == 8 || t->gc == 4 || t->gc == 2;
 }
 
+// Per-block ALU version: four lanes per (token, block); fp8: E4M3 codes instead of E2M1.
+batq_status launch_quantize_small(const batq_transform* t, const void* x, int64_t s, int64_t n, int64_t ld, void* codes,
+                                  void* scales, int32_t layout, float* debug_out, cudaStream_t stream,
+                                  uint32_t* zero_words, int32_t n_zero_words, bool fp8) {
+  QuantSmallParams q{};
+  q.x = static_cast<const uint16_t*>(x);
+  q.ld = ld;
+  q.s = static_cast<int32_t>(s);
+  q.n = static_cast<int32_t>(n);
+  q.k = static_cast<int32_t>(n / 32);
+  if (t != nullptr) {
+    q.left = t->d_left; q.right = t->d_right;
+    q.left_stride = t->left_stride; q.right_stride = t->right_stride;
+    q.clip_lo = t->d_clip_lo; q.clip_hi = t->d_clip_hi;
+  }
+  q.codes = static_cast<uint8_t*>(codes);
+  q.scales = static_cast<uint8_t*>(scales);
+  q.sf_layout = layout;
+  q.sf_katoms = katoms_of(q.k);
+  q.debug_out = debug_out;
+  q.zero_words = zero_words;
+  q.n_zero_words = n_zero_words;
+  q.bf16_mid = t != nullptr && t->bf16_mid ? 1 : 0;
+  // Launched as a programmatic dependent of whatever precedes it on the stream (in a decode loop
+  // the GEMM of the layer before): it is scheduled early and waits inside the kernel.
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(static_cast<unsigned>((s * q.k + 31) / 32));  // four lanes per (token, block)
+  cfg.blockDim = dim3(128);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const int gc = t != nullptr ? t->gc : 8;
+  const bool dbg = debug_out != nullptr;
+  cudaError_t e;
+#define BATQ_QS(GC) (fp8   ? cudaLaunchKernelEx(&cfg, quantize_act_small_kernel<false, GC, true>, q) \
+                     : dbg ? cudaLaunchKernelEx(&cfg, quantize_act_small_kernel<true, GC>, q)       \
+                           : cudaLaunchKernelEx(&cfg, quantize_act_small_kernel<false, GC>, q))
+  e = gc == 8 ? BATQ_QS(8) : gc == 4 ? BATQ_QS(4) : BATQ_QS(2);
+#undef BATQ_QS
+  if (e != cudaSuccess) { cudaGetLastError(); return BATQ_ERR_CUDA; }
+  return BATQ_OK;
+}
+
+// Up to how many tokens the per-block ALU kernel is the quicker one (tensor cores above).  Narrower
+// right factors cost the four lanes more work per block (8 x 4: 2.0 us at 16 tokens and 4.5 us at
+// 128 for n = 4096; 16 x 2: 2.9 and 7.8 us; the tensor-core kernel 4.0-4.2 us throughout).
+int64_t small_quant_limit(const batq_transform* t) {
+  if (t == nullptr || t->gc == 8) return kSmallQuantAuto;
+  return t->gc == 4 ? 64 : t->gc == 2 ? 32 : 0;
+}
+
+// MXFP8 quantiser: the same two kernels, the same line between them.
+batq_status launch_quantize_fp8(const batq_transform* t, const void* x, int64_t s, int64_t n, int64_t ld, void* codes,
+                                void* scales, int32_t layout, cudaStream_t stream, int sm_count) {
+  const int force_q = g_force_quantizer.load(std::memory_order_relaxed);
+  if (force_q != 2 && alu_small_geometry(t) && (force_q == 3 || s <= small_quant_limit(t)))
+    return launch_quantize_small(t, x, s, n, ld, codes, scales, layout, nullptr, stream, nullptr, 0, true);
+  return launch_quantize_tc(t, x, s, n, ld, codes, scales, layout, nullptr, stream, sm_count, true);
+}
+
 batq_status launch_quantize(const batq_transform* t, const void* x, int64_t s, int64_t n, int64_t ld, void* codes,
                             void* scales, int32_t layout, float* debug_out, cudaStream_t stream,
                             uint32_t* zero_words = nullptr, int32_t n_zero_words = 0) {
@@ -398,10 +469,7 @@ batq_status launch_quantize(const batq_transform* t, const void* x, int64_t s, i
   const bool mid = t != nullptr && t->bf16_mid;   // needs the factored form: the ALU kernels (4 x 8 only, checked when it is set)
   const bool small_path = n_zero_words > 0;  // in front of the small-s GEMM (its tickets to clear)
   const int force_q = g_force_quantizer.load(std::memory_order_relaxed);
-  // Narrower right factors cost the four lanes more work per block (8 x 4: 2.0 us at 16 tokens and
-  // 4.5 us at 128 for n = 4096; 16 x 2: 2.9 and 7.8 us; the tensor-core kernel 4.0-4.2 us throughout).
-  const int64_t small_limit = stream_ok ? kSmallQuantAuto : (t->gc == 4 ? 64 : 32);
-  const bool want_small = force_q == 3 || (force_q == 0 && (s <= small_limit || (stream_ok && small_path && s <= kSmallSMax)));
+  const bool want_small = force_q == 3 || (force_q == 0 && (s <= small_quant_limit(t) || (stream_ok && small_path && s <= kSmallSMax)));
   const bool use_tc = !small_ok || (!stream_ok && !want_small) ||
                       (!mid && !small_path && t != nullptr && (force_q == 2 || (force_q == 0 && s > kSmallQuantAuto)));
   if (use_tc) {
@@ -412,51 +480,10 @@ batq_status launch_quantize(const batq_transform* t, const void* x, int64_t s, i
     }
     return launch_quantize_tc(t, x, s, n, ld, codes, scales, layout, debug_out, stream, info->sm_count);
   }
-  // A handful of tokens: the ring of the streaming kernel below is all latency there; one thread
-  // per (token, block) with everything loaded up front is quicker.
-  if (want_small) {
-    QuantSmallParams q{};
-    q.x = static_cast<const uint16_t*>(x);
-    q.ld = ld;
-    q.s = static_cast<int32_t>(s);
-    q.n = static_cast<int32_t>(n);
-    q.k = static_cast<int32_t>(n / 32);
-    if (t != nullptr) {
-      q.left = t->d_left; q.right = t->d_right;
-      q.left_stride = t->left_stride; q.right_stride = t->right_stride;
-      q.clip_lo = t->d_clip_lo; q.clip_hi = t->d_clip_hi;
-    }
-    q.codes = static_cast<uint8_t*>(codes);
-    q.scales = static_cast<uint8_t*>(scales);
-    q.sf_layout = layout;
-    q.sf_katoms = katoms_of(q.k);
-    q.debug_out = debug_out;
-    q.zero_words = zero_words;
-    q.n_zero_words = n_zero_words;
-    q.bf16_mid = mid ? 1 : 0;
-    // Launched as a programmatic dependent of whatever precedes it on the stream (in a decode loop
-    // the GEMM of the layer before): it is scheduled early and waits inside the kernel.
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(static_cast<unsigned>((s * q.k + 31) / 32));  // four lanes per (token, block)
-    cfg.blockDim = dim3(128);
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    const int gc = t != nullptr ? t->gc : 8;
-    const bool dbg = debug_out != nullptr;
-    cudaError_t e;
-    if (gc == 8)      e = dbg ? cudaLaunchKernelEx(&cfg, quantize_act_small_kernel<true, 8>, q)
-                              : cudaLaunchKernelEx(&cfg, quantize_act_small_kernel<false, 8>, q);
-    else if (gc == 4) e = dbg ? cudaLaunchKernelEx(&cfg, quantize_act_small_kernel<true, 4>, q)
-                              : cudaLaunchKernelEx(&cfg, quantize_act_small_kernel<false, 4>, q);
-    else              e = dbg ? cudaLaunchKernelEx(&cfg, quantize_act_small_kernel<true, 2>, q)
-                              : cudaLaunchKernelEx(&cfg, quantize_act_small_kernel<false, 2>, q);
-    if (e != cudaSuccess) { cudaGetLastError(); return BATQ_ERR_CUDA; }
-    return BATQ_OK;
-  }
+  // A handful of tokens: the ring of the streaming kernel below is all latency there; four lanes
+  // per (token, block) with everything loaded up front are quicker.
+  if (want_small)
+    return launch_quantize_small(t, x, s, n, ld, codes, scales, layout, debug_out, stream, zero_words, n_zero_words, false);
   QuantActParams p{};
   p.x = static_cast<const uint16_t*>(x);
   p.ld = ld;
@@ -984,10 +1011,11 @@ bool cluster_reduce_ok(int64_t tiles, int sp, int64_t slots, int64_t s) {
 // time = waves x (K-steps per CTA + fixed cost) + a reduction term that grows with the splits,
 // plus the round trip through scratch and tickets where the cluster reduction does not apply
 // (all in units of one K-step of streaming, about 0.5 us).
-int pick_splits(int64_t m, int64_t n, int64_t s, int sm_count) {
+// `cluster_only`: no scratch to fall back to, only splits that meet as a cluster (MXFP8 activations).
+int pick_splits(int64_t m, int64_t n, int64_t s, int sm_count, bool cluster_only = false) {
   const int k_steps = static_cast<int>((n + 255) / 256);
   const int force_splits = g_force_splits.load(std::memory_order_relaxed);
-  if (force_splits > 0) return std::min(std::min(force_splits, k_steps), kMaxSplits);
+  if (force_splits > 0) return std::min(std::min(force_splits, k_steps), cluster_only ? 8 : kMaxSplits);
   const int64_t tiles = (m + 127) / 128;
   const int64_t slots = 2 * static_cast<int64_t>(sm_count > 0 ? sm_count : 148);
   int best = 1;
@@ -995,7 +1023,10 @@ int pick_splits(int64_t m, int64_t n, int64_t s, int sm_count) {
   for (int sp = 1; sp <= std::min(k_steps, kMaxSplits); ++sp) {
     const int64_t waves = (tiles * sp + slots - 1) / slots;
     double cost = static_cast<double>(waves) * ((k_steps + sp - 1) / sp + 3.0) + 0.15 * sp;
-    if (sp > 1 && !cluster_reduce_ok(tiles, sp, slots, s)) cost += 2.0;
+    if (sp > 1 && !cluster_reduce_ok(tiles, sp, slots, s)) {
+      if (cluster_only) continue;
+      cost += 2.0;
+    }
     if (cost < best_cost - 1e-9) { best_cost = cost; best = sp; }
   }
   return best;
@@ -1021,13 +1052,24 @@ SmallScratch small_scratch(const batq_weight* w, int64_t s) {
   return sc;
 }
 
-template <int NTOK, bool BF>
+// The same for the W4A8 GEMM, whose callers hand over no scratch: the splits meet as a cluster or
+// there is one.
+SmallScratch small_scratch_a8(const batq_weight* w, int64_t s) {
+  SmallScratch sc{};
+  sc.ntok = small_ntok(s);
+  sc.splits = pick_splits(w->m, w->n, s, w->sm_count, true);
+  sc.tiles = (w->m + 127) / 128;
+  sc.cluster = sc.splits > 1;
+  return sc;
+}
+
+template <int NTOK, bool BF, bool A8>
 cudaError_t launch_small_kernel(dim3 grid, cudaStream_t stream, bool dependent, const CUtensorMap& tw,
                                 const CUtensorMap& tx, const SmallParams& p) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(kSmallThreads);
-  cfg.dynamicSmemBytes = SmallCfg<NTOK>::kSmemBytes;
+  cfg.dynamicSmemBytes = SmallCfg<NTOK, A8>::kSmemBytes;
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
   int na = 0;
@@ -1045,21 +1087,21 @@ cudaError_t launch_small_kernel(dim3 grid, cudaStream_t stream, bool dependent, 
   }
   cfg.attrs = attr;
   cfg.numAttrs = na;
-  return cudaLaunchKernelEx(&cfg, gemm_small_s_kernel<NTOK, BF>, tw, tx, p);
+  return cudaLaunchKernelEx(&cfg, gemm_small_s_kernel<NTOK, BF, A8>, tw, tx, p);
 }
 
 // `dependent`: the kernel directly before this one on the stream is the activation quantiser
 // (which releases its dependents early); the weight stream then starts while it still runs.
 batq_status launch_gemm_small(const void* x_codes, const void* x_sf, const batq_weight* w, int64_t s, void* y,
                               int32_t y_dtype, int64_t ldy, uint8_t* scratch, const SmallScratch& sc,
-                              cudaStream_t stream, bool dependent) {
+                              cudaStream_t stream, bool dependent, bool a8 = false) {
   int dev;
   const DeviceInfo* info;
   batq_status st = device_setup(&dev, &info);
   if (st != BATQ_OK) return st;
   if (w->device != dev) return BATQ_ERR_CUDA;
   CUtensorMap tmap_x;
-  st = make_codes_tmap(&tmap_x, x_codes, s, w->n / 2, sc.ntok);
+  st = make_codes_tmap(&tmap_x, x_codes, s, a8 ? w->n : w->n / 2, sc.ntok);
   if (st != BATQ_OK) return st;
   SmallParams p{};
   p.sfx = static_cast<const uint8_t*>(x_sf);
@@ -1067,7 +1109,7 @@ batq_status launch_gemm_small(const void* x_codes, const void* x_sf, const batq_
   p.s = static_cast<int32_t>(s);
   p.m = static_cast<int32_t>(w->m);
   p.katoms = w->katoms;
-  p.k_steps = static_cast<int32_t>((w->n + 255) / 256);
+  p.k_steps = static_cast<int32_t>(a8 ? w->n / kW4A8KElems : (w->n + 255) / 256);
   p.splits = sc.splits;
   p.y = y;
   p.ldy = ldy;
@@ -1077,13 +1119,18 @@ batq_status launch_gemm_small(const void* x_codes, const void* x_sf, const batq_
   const dim3 grid(static_cast<unsigned>(sc.tiles), static_cast<unsigned>(sc.splits));
   const bool bf = y_dtype == BATQ_BF16;
   cudaError_t e;
-#define BATQ_SMALL(NT) (bf ? launch_small_kernel<NT, true>(grid, stream, dependent, w->tmap_b128, tmap_x, p) \
-                           : launch_small_kernel<NT, false>(grid, stream, dependent, w->tmap_b128, tmap_x, p))
+#define BATQ_SMALL4(NT) (bf ? launch_small_kernel<NT, true, false>(grid, stream, dependent, w->tmap_b128, tmap_x, p) \
+                            : launch_small_kernel<NT, false, false>(grid, stream, dependent, w->tmap_b128, tmap_x, p))
+#define BATQ_SMALL8(NT) (bf ? launch_small_kernel<NT, true, true>(grid, stream, dependent, w->tmap_u4_128, tmap_x, p) \
+                            : launch_small_kernel<NT, false, true>(grid, stream, dependent, w->tmap_u4_128, tmap_x, p))
+#define BATQ_SMALL(NT) (a8 ? BATQ_SMALL8(NT) : BATQ_SMALL4(NT))
   if (sc.ntok == 16) e = BATQ_SMALL(16);
   else if (sc.ntok == 32) e = BATQ_SMALL(32);
   else if (sc.ntok == 64) e = BATQ_SMALL(64);
   else e = BATQ_SMALL(128);
 #undef BATQ_SMALL
+#undef BATQ_SMALL4
+#undef BATQ_SMALL8
   if (e != cudaSuccess) { cudaGetLastError(); return BATQ_ERR_CUDA; }
   return BATQ_OK;
 }
@@ -1279,6 +1326,16 @@ batq_status launch_gemm_w4a8(const void* x_codes8, const void* x_sf, const batq_
   if (st != BATQ_OK) return st;
   if (w->device != dev) return BATQ_ERR_CUDA;
   if (!w->has_u4) return BATQ_ERR_UNSUPPORTED;
+  // A handful of tokens: bound by streaming the weights, which the swapped-operand kernel does over
+  // the whole chip whatever the number of features, its K splits meeting as clusters.  Whole layer,
+  // back to back, swapped operands against one CTA per tile behind the same quantiser: at 8 tokens
+  // 7.0 / 11.5 us (4096 -> 6144), 6.1 / 11.2 (4096 -> 4096), 14.4 / 25.5 (4096 -> 28672), 10.7 / 36
+  // (14336 -> 4096).  The reduction grows with the tokens: 12.1 / 12.0 us at 64 and 15.2 / 13.0 at
+  // 96 on 4096 -> 6144, but 22.7 / 22.9 at 96 and 23.5 / 23.7 at 128 on 4096 -> 28672, 23.9 / 37 at
+  // 128 on 14336 -> 4096, so above 64 tokens only layers of 40 M weights and more take it.
+  if (g_force_gemm_kernel.load(std::memory_order_relaxed) == 0 &&
+      (s <= 64 || (s <= kSmallSMax && w->m * w->n >= 40000000)))
+    return launch_gemm_small(x_codes8, x_sf, w, s, y, y_dtype, ldy, nullptr, small_scratch_a8(w, s), stream, dependent, true);
   const bool bf = y_dtype == BATQ_BF16;
   CUtensorMap tmap_a, tmap_y;
   std::memset(&tmap_y, 0, sizeof(tmap_y));
@@ -1553,8 +1610,8 @@ batq_status batq_quantize_act_mxfp8(const batq_transform* t, const void* x_bf16,
   st = device_setup(&dev, &info);
   if (st != BATQ_OK) return st;
   if (t->device != dev) return BATQ_ERR_CUDA;
-  return launch_quantize_tc(t, x_bf16, s, n, ld, codes, scales, scale_layout, nullptr,
-                            static_cast<cudaStream_t>(stream), info->sm_count, true);
+  return launch_quantize_fp8(t, x_bf16, s, n, ld, codes, scales, scale_layout, static_cast<cudaStream_t>(stream),
+                             info->sm_count);
 }
 
 batq_status batq_debug_transform_clip_f32(const batq_transform* t, const void* x_bf16, int64_t s, int64_t n,
@@ -1777,7 +1834,7 @@ batq_status batq_linear_w4a8(const batq_transform* t, const batq_weight* w, cons
   uint8_t* codes = static_cast<uint8_t*>(workspace);
   uint8_t* sf = codes + round_up(static_cast<size_t>(s * w->n), 1024);
   cudaStream_t cs = static_cast<cudaStream_t>(stream);
-  st = launch_quantize_tc(t, x_bf16, s, w->n, ld, codes, sf, BATQ_SF_MMA, nullptr, cs, info->sm_count, true);
+  st = launch_quantize_fp8(t, x_bf16, s, w->n, ld, codes, sf, BATQ_SF_MMA, cs, info->sm_count);
   if (st != BATQ_OK) return st;
   return launch_gemm_w4a8(codes, sf, w, s, y, y_dtype, ldy, cs, true);
 }

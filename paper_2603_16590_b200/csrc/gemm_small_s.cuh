@@ -27,20 +27,27 @@
 #include <cuda_bf16.h>
 
 #include "gemm_mxfp4.cuh"
+#include "gemm_w4a8.cuh"
 #include "ptx.cuh"
 
 namespace batq {
 
 constexpr int kSmallThreads = 192;
 
-template <int NTOK>
+// A8 = false: MXFP4 activations (kind::mxf4, a K-step of 256 elements = 128 packed bytes per row).
+// A8 = true: MXFP8 (E4M3) activations (kind::mxf8f6f4, a K-step of 128 elements): the packed weight
+// codes are widened to one byte each by the TMA unit on their way into shared memory, so a stage
+// of 16 KiB of weights is 8 KiB of the stream from HBM.
+template <int NTOK, bool A8 = false>
 struct SmallCfg {
   static constexpr int kWBytes = 128 * kBKBytes;     // 16 KiB of weight codes per K-step
   static constexpr int kXBytes = NTOK * kBKBytes;    // activation codes
-  static constexpr int kSfBytes = 1024;              // two 512-byte scale atoms (8 blocks), per operand
+  static constexpr int kSfBytes = A8 ? 512 : 1024;   // scale atoms of a K-step (4 blocks each), per operand
   static constexpr int kStageBytes = kWBytes + kXBytes + 2 * kSfBytes;
+  static constexpr int kTxBytes = kStageBytes - (A8 ? kWBytes / 2 : 0);  // a widening load reports the packed bytes
   static constexpr int kStages = (NTOK == 128) ? 3 : (NTOK == 64) ? 4 : 5;
-  static constexpr int kSfColsPerStage = 16;         // W: 2 atoms x 4 columns, X: 2 atoms x 4 columns
+  static constexpr int kSfCols = A8 ? 4 : 8;         // tensor-memory columns of one operand's scales of a K-step
+  static constexpr int kSfColsPerStage = 2 * kSfCols;
   static constexpr int kTmemCols = (NTOK == 128) ? 256 : 128;
   // Receive buffer of the push reduction (16-token tile only): [source split][ceil(s / splits)][128] fp32,
   // at most (16 + 7 - 1) / 7 * 7 = 21 token slots of 512 bytes.  It is apart from the ring: a faster
@@ -54,13 +61,20 @@ struct SmallCfg {
   static_assert(kStageBytes % 1024 == 0, "stage alignment");
 };
 
+// Instruction descriptor of kind::mxf8f6f4 with the operands swapped: A = E2M1 weights (format 5),
+// B = E4M3 activations (format 0); the fields as in mxf8f6f4_idesc_e4m3_e2m1.
+__host__ __device__ constexpr uint32_t mxf8f6f4_idesc_e2m1_e4m3(int M, int N) {
+  return (5u << 7) | (0u << 10) | (static_cast<uint32_t>(N >> 3) << 17) | (1u << 23) |
+         (static_cast<uint32_t>(M >> 4) << 24);
+}
+
 struct SmallParams {
   const uint8_t* sfx;    // activation scales, BATQ_SF_MMA layout (one 128-row tile)
   const uint8_t* sfw;    // weight scales, BATQ_SF_MMA layout
   int32_t s;             // tokens (<= NTOK)
   int32_t m;             // weight rows = output features
   int32_t katoms;        // 2*ceil(k/8)
-  int32_t k_steps;       // ceil(n / 256)
+  int32_t k_steps;       // ceil(n / 256); n / 128 with MXFP8 activations
   int32_t splits;        // gridDim.y
   void* y;               // [s x m] fp32 or bf16, row stride ldy
   int64_t ldy;
@@ -85,11 +99,13 @@ __device__ __forceinline__ void named_barrier_sync(int id, int threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 
-template <int NTOK, bool OUT_BF16>
+template <int NTOK, bool OUT_BF16, bool A8>
 __global__ void __launch_bounds__(kSmallThreads, 2)
 gemm_small_s_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_x,
                     const SmallParams p) {
-  using Cfg = SmallCfg<NTOK>;
+  using Cfg = SmallCfg<NTOK, A8>;
+  constexpr int kStepX = 128;   // K coordinate of a step in either tensor map: 128 packed bytes, 128 8-bit codes or 128 widened 4-bit codes
+  static_assert(kStepX == kBKBytes, "one swizzle row per K-step");
   extern __shared__ uint8_t small_smem_raw[];
   __shared__ __align__(8) uint64_t full_bar[Cfg::kStages];
   __shared__ __align__(8) uint64_t empty_bar[Cfg::kStages];
@@ -141,15 +157,15 @@ gemm_small_s_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
     auto load_w = [&](int stage, int kt) {
       const uint32_t st = smem_base + stage * Cfg::kStageBytes;
       const uint32_t bar = smem_u32(&full_bar[stage]);
-      mbar_arrive_expect_tx(bar, Cfg::kStageBytes);
-      tma_load_2d(st, &tmap_w, kt * kBKBytes, rt * 128, bar);
-      bulk_g2s(st + Cfg::kWBytes + Cfg::kXBytes, sfw_src + static_cast<int64_t>(kt) * 1024, 1024, bar);
+      mbar_arrive_expect_tx(bar, Cfg::kTxBytes);
+      tma_load_2d(st, &tmap_w, kt * kStepX, rt * 128, bar);
+      bulk_g2s(st + Cfg::kWBytes + Cfg::kXBytes, sfw_src + static_cast<int64_t>(kt) * Cfg::kSfBytes, Cfg::kSfBytes, bar);
     };
     auto load_x = [&](int stage, int kt) {
       const uint32_t st = smem_base + stage * Cfg::kStageBytes;
       const uint32_t bar = smem_u32(&full_bar[stage]);
-      tma_load_2d(st + Cfg::kWBytes, &tmap_x, kt * kBKBytes, 0, bar);
-      bulk_g2s(st + Cfg::kWBytes + Cfg::kXBytes + Cfg::kSfBytes, p.sfx + static_cast<int64_t>(kt) * 1024, 1024, bar);
+      tma_load_2d(st + Cfg::kWBytes, &tmap_x, kt * kStepX, 0, bar);
+      bulk_g2s(st + Cfg::kWBytes + Cfg::kXBytes + Cfg::kSfBytes, p.sfx + static_cast<int64_t>(kt) * Cfg::kSfBytes, Cfg::kSfBytes, bar);
     };
     // Weights first: they do not depend on the kernel that quantises the activations.
     const int prefill = min(n_steps, Cfg::kStages);
@@ -185,7 +201,7 @@ gemm_small_s_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
     }
   } else if (warp == 1) {
     // ---------------------------------------------------------------- MMA issuer
-    constexpr uint32_t idesc0 = mxf4_idesc(128, NTOK);
+    constexpr uint32_t idesc0 = A8 ? mxf8f6f4_idesc_e2m1_e4m3(128, NTOK) : mxf4_idesc(128, NTOK);
     constexpr uint32_t idesc1 = idesc0 | (2u << 29) | (2u << 4);  // scale byte pair 2 instead of 0
     const uint32_t smem_base = smem_u32(smem);
     const uint64_t w_desc0 = make_smem_desc(smem_base, 16, 1024, 2);
@@ -203,14 +219,19 @@ gemm_small_s_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
       const uint64_t xdesc = wdesc + (Cfg::kWBytes >> 4);
       const uint64_t sfd = sf_desc0 + soff;
       const uint32_t sfw_col = sf_tmem0 + stage * Cfg::kSfColsPerStage;
-      const uint32_t sfx_col = sfw_col + 8;
+      const uint32_t sfx_col = sfw_col + Cfg::kSfCols;
       if (elect_one()) {
-        tc_cp_32x128b_warpx4(sfw_col, sfd);
-        tc_cp_32x128b_warpx4(sfw_col + 4, sfd + 32);
-        tc_cp_32x128b_warpx4(sfx_col, sfd + 64);
-        tc_cp_32x128b_warpx4(sfx_col + 4, sfd + 96);
+#pragma unroll
+        for (int a = 0; a < 2 * Cfg::kSfBytes / 512; ++a)   // W's atoms, then X's, side by side in both memories
+          tc_cp_32x128b_warpx4(sfw_col + 4 * a, sfd + 32 * a);
 #pragma unroll
         for (int kb = 0; kb < 4; ++kb) {
+          if (A8) {   // 32 elements per MMA: byte kb of the scale column
+            const uint32_t b = static_cast<uint32_t>(kb);
+            tc_mma_mxf8f6f4(tmem_base, wdesc + 2 * kb, xdesc + 2 * kb, idesc0 | (b << 29) | (b << 4), sfw_col | (b << 30),
+                            sfx_col | (b << 30), (i | kb) != 0 ? 1u : 0u);
+            continue;
+          }
           const uint32_t c = kb >> 1;
           const uint32_t sfid = (kb & 1) * 2;
           tc_mma_mxf4(tmem_base, wdesc + 2 * kb, xdesc + 2 * kb, (kb & 1) ? idesc1 : idesc0,

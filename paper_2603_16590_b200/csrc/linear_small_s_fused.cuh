@@ -24,6 +24,7 @@
 #include "gemm_small_s.cuh"
 #include "ptx.cuh"
 #include "quantize_act.cuh"
+#include "quantize_act_tc.cuh"
 
 namespace batq {
 
@@ -190,6 +191,17 @@ __device__ __forceinline__ void quad_encode(const float (&o)[8], float amax, uin
   sbyte = static_cast<uint32_t>(sb);
 }
 
+// The same for MXFP8 (E4M3 codes, e = floor(log2 amax) - 8): two words of codes.
+__device__ __forceinline__ void quad_encode8(const float (&o)[8], float amax, uint32_t (&cw)[2], uint32_t& sbyte) {
+  const int ef = static_cast<int>(__float_as_uint(amax) >> 23);
+  const int sb = max(ef - 8, 0);
+  const float inv = __uint_as_float(static_cast<uint32_t>(254 - sb) << 23);
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+    cw[h] = e4m3x4_pack(o[4 * h] * inv, o[4 * h + 1] * inv, o[4 * h + 2] * inv, o[4 * h + 3] * inv);
+  sbyte = static_cast<uint32_t>(sb);
+}
+
 // ---------------------------------------------------------------------------------------------
 // Stages 1+2 alone for a handful of tokens: four lanes per (token, block), the factors requested
 // before the wait for the previous grid and x right after it, no shared-memory ring -- a launch of
@@ -207,7 +219,7 @@ struct QuantSmallParams {
   int32_t right_stride;
   const float* clip_lo;  // [k] or NULL
   const float* clip_hi;
-  uint8_t* codes;        // [s x n/2]
+  uint8_t* codes;        // [s x n/2], FP8: [s x n]
   uint8_t* scales;
   int32_t sf_layout;     // BATQ_SF_ROWMAJOR / BATQ_SF_MMA
   int32_t sf_katoms;
@@ -217,7 +229,7 @@ struct QuantSmallParams {
   int32_t bf16_mid;      // != 0: both contractions of the transform store their result as bf16
 };
 
-template <bool DEBUG_OUT, int GC>
+template <bool DEBUG_OUT, int GC, bool FP8 = false>
 __global__ void __launch_bounds__(128) quantize_act_small_kernel(const QuantSmallParams p) {
   grid_launch_dependents();
   const int lane = threadIdx.x & 31;
@@ -246,9 +258,16 @@ __global__ void __launch_bounds__(128) quantize_act_small_kernel(const QuantSmal
     dst[1] = make_float4(o[4], o[5], o[6], o[7]);
     return;
   }
-  uint32_t cw, sbyte;
-  quad_encode(o, amax, cw, sbyte);
-  *reinterpret_cast<uint32_t*>(p.codes + row * (p.n / 2) + static_cast<int64_t>(j) * 16 + r * 4) = cw;
+  uint32_t sbyte;
+  if (FP8) {
+    uint32_t cw[2];
+    quad_encode8(o, amax, cw, sbyte);
+    *reinterpret_cast<uint2*>(p.codes + row * p.n + static_cast<int64_t>(j) * 32 + r * 8) = make_uint2(cw[0], cw[1]);
+  } else {
+    uint32_t cw;
+    quad_encode(o, amax, cw, sbyte);
+    *reinterpret_cast<uint32_t*>(p.codes + row * (p.n / 2) + static_cast<int64_t>(j) * 16 + r * 4) = cw;
+  }
   if (r != 0) return;
   if (p.sf_layout == 0) {
     p.scales[row * p.k + j] = static_cast<uint8_t>(sbyte);

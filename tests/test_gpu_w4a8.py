@@ -71,6 +71,52 @@ def test_w4a8_gemm_vs_oracle_same_codes(batq, gkernel, S, M, N, bn):
     assert np.max(np.abs(got - Y) / (Sabs + 1e-30)) < 1e-5
 
 
+@pytest.mark.parametrize("splits", [0, 1, 2, 3, 7, 8])
+@pytest.mark.parametrize("S,M,N", [(1, 8, 128), (16, 264, 1152), (17, 136, 1024), (33, 128, 2176), (64, 520, 896)])
+def test_w4a8_few_tokens_gemm_vs_oracle_same_codes(batq, S, M, N, splits):
+    """The swapped-operand kernel: both sides of every token tile (16, 32, 64), part-filled row tiles,
+    K-step counts that the splits divide and do not divide (fewer K-steps than splits: fewer splits)."""
+    batq.batq_debug_force_small_s_splits(splits)
+    try:
+        got, Y, Sabs = _gemm_case(batq, S, M, N, 2600 + S)
+    finally:
+        batq.batq_debug_force_small_s_splits(0)
+    # exact products, fp32 accumulation of N terms in any order: below N 2^-24 Sabs < 1.4e-4, in fact < 1e-5
+    assert np.max(np.abs(got - Y) / (Sabs + 1e-30)) < 1e-5
+
+
+def test_w4a8_128_token_tile_of_a_large_layer(batq):
+    """The 128-token tile, which automatic dispatch keeps for layers of 40 M weights and more."""
+    got, Y, Sabs = _gemm_case(batq, 128, 5008, 8192, 2700)
+    assert np.max(np.abs(got - Y) / (Sabs + 1e-30)) < 1e-5
+
+
+@pytest.mark.parametrize("layout", [0, 1])
+@pytest.mark.parametrize("gr,gc", [(4, 8), (8, 4), (16, 2)])
+@pytest.mark.parametrize("S,N", [(1, 32), (5, 96), (32, 1056), (33, 256)])
+def test_mxfp8_per_block_quantiser_vs_tensor_cores(batq, S, N, gr, gc, layout):
+    """The ALU quantiser's codes and scale bytes against the tensor-core kernel's: fp32 sums in another
+    order, so a code may sit on the other side of a rounding boundary (E4M3 half steps are at least
+    2^-5 of a code's value, the sums differ by < 2^-20 of theirs: well below 1e-3 of the codes)."""
+    t = synth.make_transform(N, 5, "naive", gr=gr, gc=gc)
+    tr = _mk(batq, t)
+    x = batq.bits_to_cuda_bf16(synth.make_activations(S, N, 77))
+    out = []
+    for mode in (2, 3):
+        batq.batq_debug_force_quantizer(mode)
+        codes = torch.full((S, N), 0xEE, dtype=torch.uint8, device="cuda")
+        sf = torch.full((batq.batq_sf_bytes(S, N, layout),), 0xEE, dtype=torch.uint8, device="cuda")
+        try:
+            batq.batq_quantize_act_mxfp8(tr, x, codes, sf, layout)
+        finally:
+            batq.batq_debug_force_quantizer(0)
+        h = sf.cpu().numpy()
+        out.append((codes.cpu().numpy().astype(np.int32), sf_mma_to_rowmajor(h, S, N // 32) if layout else h.reshape(S, N // 32)))
+    assert np.array_equal(out[0][1], out[1][1])
+    differ = out[0][0] != out[1][0]
+    assert differ.mean() <= 1e-3 and np.abs(out[0][0] - out[1][0]).max() <= 1
+
+
 @pytest.mark.parametrize("bn", [64, 128, 192, 256, 320, 384, 448])
 def test_w4a8_scale_layout_localising_case(batq, gkernel, bn):
     """Constant codes and a distinct power-of-two scale per (row, block) on both sides: a mistake in
