@@ -27,6 +27,7 @@
 #include "prepare_weight.cuh"
 #include "quantize_act.cuh"
 #include "quantize_act_tc.cuh"
+#include "quantize_act_warp.cuh"
 
 using namespace batq;
 
@@ -324,7 +325,7 @@ batq_status check_x(const void* x, int64_t s, int64_t n, int64_t ld) {
 
 constexpr int64_t kSmallSMax = 128;       // the swapped-operand split-K GEMM takes up to this many tokens
 constexpr int64_t kSmallQuantAuto = 128;  // per-block ALU quantiser up to here, tensor cores above (4.0 us against 1.7-3.0 us back to back at n = 4096)
-std::atomic<int> g_force_quantizer{0};  // tuning hook: 0 = automatic, 1 = ALU (Kronecker form), 2 = tensor cores (dense form)
+std::atomic<int> g_force_quantizer{0};  // tuning hook: 0 = automatic, 1 = ALU (Kronecker form, streaming), 2 = tensor cores (dense form), 3 = ALU per block, 4 = ALU, thread per item
 
 // Tensor-core version: 128-token x 4-block units.
 batq_status launch_quantize_tc(const batq_transform* t, const void* x, int64_t s, int64_t n, int64_t ld, void* codes,
@@ -434,7 +435,53 @@ batq_status launch_quantize_small(const batq_transform* t, const void* x, int64_
   return BATQ_OK;
 }
 
-// Up to how many tokens the per-block ALU kernel is the quicker one (tensor cores above).  Narrower
+// One thread per (token, block), straight from and to global memory (4 x 8 and 8 x 4 factors).
+batq_status launch_quantize_warp(const batq_transform* t, const void* x, int64_t s, int64_t n, int64_t ld, void* codes,
+                                 void* scales, int32_t layout, cudaStream_t stream, int sm_count, uint32_t* zero_words,
+                                 int32_t n_zero_words, bool fp8) {
+  QuantWarpParams q{};
+  q.x = static_cast<const uint16_t*>(x);
+  q.ld = ld;
+  q.s = s;
+  q.n = static_cast<int32_t>(n);
+  q.k = static_cast<int32_t>(n / 32);
+  q.left = t->d_left; q.right = t->d_right;
+  q.left_stride = t->left_stride; q.right_stride = t->right_stride;
+  q.clip_lo = t->d_clip_lo;
+  q.clip_hi = t->d_clip_hi;
+  q.codes = static_cast<uint8_t*>(codes);
+  q.scales = static_cast<uint8_t*>(scales);
+  q.sf_layout = layout;
+  q.sf_katoms = katoms_of(q.k);
+  q.zero_words = zero_words;
+  q.n_zero_words = n_zero_words;
+  q.n_tiles = static_cast<int32_t>((s + kQwRows - 1) / kQwRows);
+  // Three CTAs fit an SM (168 registers a thread): where there are more tiles than that, a CTA keeps
+  // its factors and walks down the rows.
+  const int strips = layout == BATQ_SF_MMA ? q.sf_katoms : (q.k + 3) / 4;
+  const int64_t chunks = std::min<int64_t>(65535, std::max(1, 3 * sm_count / strips));
+  q.tiles_per_cta = static_cast<int32_t>((q.n_tiles + chunks - 1) / chunks);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(static_cast<unsigned>(strips), static_cast<unsigned>((q.n_tiles + q.tiles_per_cta - 1) / q.tiles_per_cta));
+  cfg.blockDim = dim3(kQwThreads);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cudaError_t e;
+#define BATQ_QW(GC) (t->has_clip ? (fp8 ? cudaLaunchKernelEx(&cfg, quantize_act_warp_kernel<GC, true, true>, q)     \
+                                        : cudaLaunchKernelEx(&cfg, quantize_act_warp_kernel<GC, true, false>, q))   \
+                                 : (fp8 ? cudaLaunchKernelEx(&cfg, quantize_act_warp_kernel<GC, false, true>, q)    \
+                                        : cudaLaunchKernelEx(&cfg, quantize_act_warp_kernel<GC, false, false>, q)))
+  e = t->gc == 8 ? BATQ_QW(8) : BATQ_QW(4);
+#undef BATQ_QW
+  if (e != cudaSuccess) { cudaGetLastError(); return BATQ_ERR_CUDA; }
+  return BATQ_OK;
+}
+
+// Up to how many tokens the per-block ALU kernel stands against the tensor-core one alone.  Narrower
 // right factors cost the four lanes more work per block (8 x 4: 2.0 us at 16 tokens and 4.5 us at
 // 128 for n = 4096; 16 x 2: 2.9 and 7.8 us; the tensor-core kernel 4.0-4.2 us throughout).
 int64_t small_quant_limit(const batq_transform* t) {
@@ -442,13 +489,25 @@ int64_t small_quant_limit(const batq_transform* t) {
   return t->gc == 4 ? 64 : t->gc == 2 ? 32 : 0;
 }
 
-// MXFP8 quantiser: the same two kernels, the same line between them.
-batq_status launch_quantize_fp8(const batq_transform* t, const void* x, int64_t s, int64_t n, int64_t ld, void* codes,
-                                void* scales, int32_t layout, cudaStream_t stream, int sm_count) {
+// (token, block) items from which the thread-per-item kernel takes over from the per-block one (2.1
+// against 2.4 us at 32 x 4096 = 4096 items, 3.1 against 2.6 at 9600, 8.0 against 4.2 at 57344).  Both
+// give the same codes; the tensor cores' fp32 sums round in another order (6.6e-8 and 8.1e-8 off the
+// exact ones), so above the limit everything stays with them although this kernel would be the quicker
+// one up to some 50000 items (200 x 4096: 3.2 against 4.4 us).
+constexpr int64_t kWarpQuantMin = 8192;
+bool warp_quant_geometry(const batq_transform* t) { return t != nullptr && !t->bf16_mid && (t->gc == 8 || t->gc == 4); }
+
+// The MXFP8 quantiser of a layer.  batq_quantize_act_mxfp8, whose bytes a caller may keep and compare,
+// has the tensor-core kernel at every size.
+batq_status launch_quantize_layer_fp8(const batq_transform* t, const void* x, int64_t s, int64_t n, int64_t ld, void* codes,
+                                      void* scales, cudaStream_t stream, int sm_count) {
   const int force_q = g_force_quantizer.load(std::memory_order_relaxed);
-  if (force_q != 2 && alu_small_geometry(t) && (force_q == 3 || s <= small_quant_limit(t)))
-    return launch_quantize_small(t, x, s, n, ld, codes, scales, layout, nullptr, stream, nullptr, 0, true);
-  return launch_quantize_tc(t, x, s, n, ld, codes, scales, layout, nullptr, stream, sm_count, true);
+  const bool small = force_q == 0 && s <= small_quant_limit(t);
+  if (warp_quant_geometry(t) && (force_q == 4 || (small && s * (n / 32) > kWarpQuantMin)))
+    return launch_quantize_warp(t, x, s, n, ld, codes, scales, BATQ_SF_MMA, stream, sm_count, nullptr, 0, true);
+  if (alu_small_geometry(t) && (force_q == 3 || small))
+    return launch_quantize_small(t, x, s, n, ld, codes, scales, BATQ_SF_MMA, nullptr, stream, nullptr, 0, true);
+  return launch_quantize_tc(t, x, s, n, ld, codes, scales, BATQ_SF_MMA, nullptr, stream, sm_count, true);
 }
 
 batq_status launch_quantize(const batq_transform* t, const void* x, int64_t s, int64_t n, int64_t ld, void* codes,
@@ -472,6 +531,9 @@ batq_status launch_quantize(const batq_transform* t, const void* x, int64_t s, i
   const bool want_small = force_q == 3 || (force_q == 0 && (s <= small_quant_limit(t) || (stream_ok && small_path && s <= kSmallSMax)));
   const bool use_tc = !small_ok || (!stream_ok && !want_small) ||
                       (!mid && !small_path && t != nullptr && (force_q == 2 || (force_q == 0 && s > kSmallQuantAuto)));
+  if (warp_quant_geometry(t) && debug_out == nullptr &&
+      (force_q == 4 || (force_q == 0 && want_small && s * (n / 32) > kWarpQuantMin)))
+    return launch_quantize_warp(t, x, s, n, ld, codes, scales, layout, stream, info->sm_count, zero_words, n_zero_words, false);
   if (use_tc) {
     if (n_zero_words > 0 &&
         cudaMemsetAsync(zero_words, 0, static_cast<size_t>(n_zero_words) * 4, stream) != cudaSuccess) {
@@ -1610,8 +1672,14 @@ batq_status batq_quantize_act_mxfp8(const batq_transform* t, const void* x_bf16,
   st = device_setup(&dev, &info);
   if (st != BATQ_OK) return st;
   if (t->device != dev) return BATQ_ERR_CUDA;
-  return launch_quantize_fp8(t, x_bf16, s, n, ld, codes, scales, scale_layout, static_cast<cudaStream_t>(stream),
-                             info->sm_count);
+  if (g_force_quantizer.load(std::memory_order_relaxed) == 3 && alu_small_geometry(t))   // tests
+    return launch_quantize_small(t, x_bf16, s, n, ld, codes, scales, scale_layout, nullptr, static_cast<cudaStream_t>(stream),
+                                 nullptr, 0, true);
+  if (g_force_quantizer.load(std::memory_order_relaxed) == 4 && warp_quant_geometry(t))
+    return launch_quantize_warp(t, x_bf16, s, n, ld, codes, scales, scale_layout, static_cast<cudaStream_t>(stream),
+                                info->sm_count, nullptr, 0, true);
+  return launch_quantize_tc(t, x_bf16, s, n, ld, codes, scales, scale_layout, nullptr,
+                            static_cast<cudaStream_t>(stream), info->sm_count, true);
 }
 
 batq_status batq_debug_transform_clip_f32(const batq_transform* t, const void* x_bf16, int64_t s, int64_t n,
@@ -1834,7 +1902,7 @@ batq_status batq_linear_w4a8(const batq_transform* t, const batq_weight* w, cons
   uint8_t* codes = static_cast<uint8_t*>(workspace);
   uint8_t* sf = codes + round_up(static_cast<size_t>(s * w->n), 1024);
   cudaStream_t cs = static_cast<cudaStream_t>(stream);
-  st = launch_quantize_fp8(t, x_bf16, s, w->n, ld, codes, sf, BATQ_SF_MMA, cs, info->sm_count);
+  st = launch_quantize_layer_fp8(t, x_bf16, s, w->n, ld, codes, sf, cs, info->sm_count);
   if (st != BATQ_OK) return st;
   return launch_gemm_w4a8(codes, sf, w, s, y, y_dtype, ldy, cs, true);
 }

@@ -117,6 +117,31 @@ def test_mxfp8_per_block_quantiser_vs_tensor_cores(batq, S, N, gr, gc, layout):
     assert differ.mean() <= 1e-3 and np.abs(out[0][0] - out[1][0]).max() <= 1
 
 
+@pytest.mark.parametrize("layout", [0, 1])
+@pytest.mark.parametrize("fp8", [False, True])
+@pytest.mark.parametrize("gr,gc", [(4, 8), (8, 4)])
+@pytest.mark.parametrize("S,N,clip", [(1, 32, True), (31, 96, False), (33, 160, True), (97, 1056, True), (1000, 8192, True)])
+def test_thread_per_item_quantiser_equals_per_block_quantiser(batq, S, N, clip, gr, gc, fp8, layout):
+    """Same fused multiply-adds in the same order: identical codes and scale bytes, at the edges of its
+    32-token tiles and 4-block strips, and where a CTA walks several tiles (the last size)."""
+    t = synth.make_transform(N, 5, "naive", clip=clip, gr=gr, gc=gc)
+    tr = _mk(batq, t)
+    x = torch.zeros((S, N + 8), dtype=torch.bfloat16, device="cuda")
+    x[:, :N] = batq.bits_to_cuda_bf16(synth.make_activations(S, N, 78))
+    out = []
+    for mode in (3, 4):
+        batq.batq_debug_force_quantizer(mode)
+        codes = torch.full((S + 1, N if fp8 else N // 2), 0xEE, dtype=torch.uint8, device="cuda")
+        sf = torch.full((batq.batq_sf_bytes(S, N, layout) + 64,), 0xEE, dtype=torch.uint8, device="cuda")
+        try:
+            (batq.batq_quantize_act_mxfp8 if fp8 else batq.batq_quantize_act)(tr, x[:, :N], codes, sf, layout)
+        finally:
+            batq.batq_debug_force_quantizer(0)
+        assert (codes[S] == 0xEE).all() and (sf[-64:] == 0xEE).all()
+        out.append((codes, sf))
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+
+
 @pytest.mark.parametrize("bn", [64, 128, 192, 256, 320, 384, 448])
 def test_w4a8_scale_layout_localising_case(batq, gkernel, bn):
     """Constant codes and a distinct power-of-two scale per (row, block) on both sides: a mistake in
