@@ -179,19 +179,14 @@ quantize_act_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_
   tc_fence_after_sync();
   const uint32_t tmem_base = tmem_base_slot;
 
-  // Units of this CTA: u0, u0 + us, ... below u1.  A CTA with many units takes a contiguous range, strip
-  // after strip, and keeps its block-matrix image; one with few takes every gridDim.x-th, strips fastest
-  // (an image, 24 KiB from L2, for nearly every unit), so that all CTAs start on their first unit alike.
-  // Few = below 16 a CTA.  Back to back, contiguous / interleaved: 333 x 14336 7.2 / 6.7 us, 2048 x 4096
-  // 8.2 / 7.7, 32768 x 128 5.7 / 5.2, 2048 x 14336 17.5 / 17.0; 32768 x 8192 on changing inputs 141 / 151.
-  const bool interleaved = p.n_units < 16 * static_cast<int64_t>(gridDim.x);
-  const int64_t us = interleaved ? gridDim.x : 1;
-  const int64_t u0 = interleaved ? blockIdx.x : p.n_units * blockIdx.x / gridDim.x;
-  const int64_t u1 = interleaved ? p.n_units : p.n_units * (blockIdx.x + 1) / gridDim.x;
-  auto unit_at = [&](int64_t u, int64_t& strip, int64_t& row_tile) {
-    if (interleaved) { row_tile = u / p.n_strips; strip = u - row_tile * p.n_strips; }
-    else { strip = u / p.n_row_tiles; row_tile = u - strip * p.n_row_tiles; }
-  };
+  // Units of this CTA: u0, u0 + us, ... below u1; unit u = strip * n_row_tiles + row_tile.  A contiguous
+  // range, so that a CTA keeps its block-matrix image; where there is one strip only there is one image
+  // anyway, and every gridDim.x-th unit is the quicker order (32768 x 128: 5.7 -> 5.2 us).  With several
+  // strips, strips fastest over the CTAs measured 0.5 us better on operands in L2 (2048 x 4096: 8.2 ->
+  // 7.7) but 1 % worse on a layer and 2-7 % worse at 32768 x 8192 on operands from HBM.
+  const int64_t us = p.n_strips == 1 ? gridDim.x : 1;
+  const int64_t u0 = p.n_strips == 1 ? blockIdx.x : p.n_units * blockIdx.x / gridDim.x;
+  const int64_t u1 = p.n_strips == 1 ? p.n_units : p.n_units * (blockIdx.x + 1) / gridDim.x;
 
   if (warp == 0) {
     // ---------------------------------------------------------------- TMA producer
@@ -203,9 +198,8 @@ quantize_act_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_
     int issued = 0;
     bool waited = false;
     for (int64_t u = u0; u < u1 && ok; u += us) {
-      int64_t strip, row_tile;
-      unit_at(u, strip, row_tile);
-      const int row0 = static_cast<int>(row_tile) * kQtRows;
+      const int64_t strip = u / p.n_row_tiles;
+      const int row0 = static_cast<int>(u - strip * p.n_row_tiles) * kQtRows;
       if (strip != cur_strip) {
         cur_strip = strip;
         const int pb = n_img & 1;
@@ -260,8 +254,7 @@ quantize_act_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_
     int it = 0;
     bool ok = true;
     for (int64_t u = u0; u < u1 && ok; u += us, ++it) {
-      int64_t strip, row_tile;
-      unit_at(u, strip, row_tile);
+      const int64_t strip = u / p.n_row_tiles;
       if (strip != cur_strip) {
         if (cur_strip >= 0 && elect_one()) tc_commit(smem_u32(&p_empty[(n_img - 1) & 1]));  // old image no longer read
         cur_strip = strip;
@@ -306,8 +299,8 @@ quantize_act_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_
     if (!DEBUG_OUT && lane == 0) {
       int it = 0;
       for (int64_t u = u0; u < u1; u += us, ++it) {
-        int64_t strip, row_tile;
-        unit_at(u, strip, row_tile);
+        const int64_t strip = u / p.n_row_tiles;
+        const int64_t row_tile = u - strip * p.n_row_tiles;
         const int sb = it % kQtOutBufs;
         if (!mbar_wait(smem_u32(&t_full[sb]), static_cast<uint32_t>(it / kQtOutBufs) & 1u, &abort_flag)) break;
         tma_store_2d(&tmap_codes, static_cast<int>(strip) * (kQtGroups * (FP8 ? 32 : 16)),
@@ -331,8 +324,8 @@ quantize_act_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_
     const int half = (qw & 7) >> 2;     // blocks 2 half and 2 half + 1 of the unit
     for (int it = grp; u0 + it * us < u1; it += 2) {
       const int64_t u = u0 + it * us;
-      int64_t strip, row_tile;
-      unit_at(u, strip, row_tile);
+      const int64_t strip = u / p.n_row_tiles;
+      const int64_t row_tile = u - strip * p.n_row_tiles;
       const int buf = it & (kQtDBufs - 1);
       bool ok = mbar_wait(smem_u32(&d_full[buf]), (it >> 2) & 1u, &abort_flag);
       ok = __all_sync(0xFFFFFFFFu, ok);
