@@ -116,7 +116,9 @@ def _ptr(t):
 
 
 def _stream():
-    return torch.cuda.current_stream().cuda_stream
+    # the handle of torch.cuda.current_stream() without the Python object around it: 0.3 us instead of 3.4
+    # of a decode call's 9.4 to 11.5
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _f32(a):
