@@ -1055,6 +1055,9 @@ batq_status launch_gemm(const void* x_codes, const void* x_sf, const batq_weight
   return BATQ_OK;
 }
 
+// Fewer 128-feature tiles than half the SMs.
+bool few_row_tiles(const batq_weight* w) { return (w->m + 127) / 128 * 2 <= w->sm_count; }
+
 // ---- small-s (decode) GEMM: split choice, scratch layout, launch -------------------------------
 std::atomic<int> g_force_splits{0};  // tuning hook: 0 = automatic
 std::atomic<int> g_small_reduce{0};  // tuning hook: 0 = automatic, 1 = always tickets, 2 = cluster whenever splits <= 8
@@ -1398,11 +1401,11 @@ batq_status launch_gemm_w4a8(const void* x_codes8, const void* x_sf, const batq_
   // the whole chip whatever the number of features, its K splits meeting as clusters.  Whole layer,
   // back to back, swapped operands against one CTA per tile behind the same quantiser: at 8 tokens
   // 7.0 / 11.5 us (4096 -> 6144), 6.1 / 11.2 (4096 -> 4096), 14.4 / 25.5 (4096 -> 28672), 10.7 / 36
-  // (14336 -> 4096).  The reduction grows with the tokens: 12.1 / 12.0 us at 64 and 15.2 / 13.0 at
-  // 96 on 4096 -> 6144, but 22.7 / 22.9 at 96 and 23.5 / 23.7 at 128 on 4096 -> 28672, 23.9 / 37 at
-  // 128 on 14336 -> 4096, so above 64 tokens only layers of 40 M weights and more take it.
+  // (14336 -> 4096); at 75 / 96 tokens 11.5 / 12.3 against 11.8 / 11.8 (4096 -> 6144) and 21.9 / 22.6
+  // against 22.1 / 22.3 (4096 -> 28672), but 18.0 against 32.8 at 96 and 21.2 against 34.4 at 128 on
+  // 14336 -> 4096: above 80 tokens only large layers with few features.
   if (g_force_gemm_kernel.load(std::memory_order_relaxed) == 0 &&
-      (s <= 64 || (s <= kSmallSMax && w->m * w->n >= 40000000)))
+      (s <= 80 || (s <= kSmallSMax && w->m * w->n >= 40000000 && few_row_tiles(w))))
     return launch_gemm_small(x_codes8, x_sf, w, s, y, y_dtype, ldy, nullptr, small_scratch_a8(w, s), stream, dependent, true);
   const bool bf = y_dtype == BATQ_BF16;
   CUtensorMap tmap_a, tmap_y;
@@ -1936,15 +1939,17 @@ batq_status batq_gemm_mxfp4_small_s(const void* x_codes, const void* x_scales_mm
   return launch_gemm_small(x_codes, x_scales_mma, w, s, y, y_dtype, ldy, sp, sc, cs, false);
 }
 
-// The whole layer takes the small-s path (per-block quantiser + swapped-operand split-K GEMM) up
-// to 32 tokens, and up to 128 where the layer is large enough for the weight stream to dominate
-// (>= 40 M weights, e.g. 4096 x 14336).  The path's cost grows with the tokens (split-K reduction
-// of tokens x 128 partial sums per CTA), while the one-CTA-per-tile GEMM behind the same per-block
-// quantiser costs about the same from 33 to 128 tokens.  Measured, 4096 -> 6144 at 32 / 48 / 64 /
-// 96 / 128 tokens: 9.0 / 10.4 / 11.4 / 14.1 / 16.0 us on the small-s path, 9.7 / 8.8 / 9.6 / 10.1 us
-// from 48 tokens on the other; 4096 -> 28672 at 96 tokens: 17.9 against 19.5 us.
+// The whole layer takes the small-s path (ALU quantiser + swapped-operand split-K GEMM) up to 32
+// tokens, up to 64 where the layer is large enough for the weight stream to dominate (>= 40 M weights),
+// and up to 128 where such a layer also has too few features to fill the chip without splitting K.
+// Measured against the one-CTA-per-tile GEMM behind the same quantiser, back to back: 4096 -> 6144 at
+// 32 / 48 / 64 tokens 7.9 / 9.0 / 9.6 us against 10.5 / 9.0 / 8.1; 4096 -> 28672 at 48 / 64 / 75 / 96 /
+// 128 tokens 14.5 / 15.8 / 17.1 / 17.9 / 18.9 against 20.9 / 17.4 / 17.1 / 17.3 / 17.7; 14336 -> 4096 at
+// 75 / 128 tokens 14.0 / 18.0 against 21.1 / 22.7.
 static bool layer_takes_small_path(const batq_weight* w, int64_t s) {
-  return s <= 32 || (s <= kSmallSMax && w->m * w->n >= 40000000);
+  if (s <= 32) return true;
+  if (s > kSmallSMax || w->m * w->n < 40000000) return false;
+  return s <= 64 || few_row_tiles(w);
 }
 
 size_t batq_linear_workspace_bytes(const batq_weight* w, int64_t s) {

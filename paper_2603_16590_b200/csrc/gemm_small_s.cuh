@@ -403,24 +403,53 @@ gemm_small_s_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
       }
     } else if (warp >= 2 && epi_ok) {
       // Reduce-scatter: CTA sp adds, in split order (deterministic), the partial sums of tokens
-      // sp, sp + splits, ... -- its own from local, the others' from distributed shared memory --
-      // and writes those tokens of y.
-      const int row = (warp & 3) * 32 + lane;
-      const int64_t mrow = static_cast<int64_t>(rt) * 128 + row;
-      const uint32_t mine = smem_u32(smem) + row * 4;
-      for (int t = sp; t < p.s; t += p.splits) {
-        float part[8];
+      // sp, sp + splits, ... -- its own from local, the others' from distributed shared memory -- and
+      // writes those tokens of y.  What a round of remote loads costs is its latency, so every warp
+      // takes tokens of its own, a lane four neighbouring rows (16-byte loads), two tokens at a time:
+      // one round for 8 of the CTA's tokens instead of one per token.  Whole layer, back to back, before
+      // and after: 4096 -> 6144 at 32 tokens 8.8 / 7.9 us (MXFP8 9.7 / 8.7), 14336 -> 4096 at 64 tokens
+      // 15.7 / 13.2 (MXFP8 17.1 / 15.8).
+      const int64_t m0 = static_cast<int64_t>(rt) * 128 + 4 * lane;
+      const uint32_t mine = smem_u32(smem) + lane * 16;
+      for (int t0 = sp + (warp & 3) * p.splits; t0 < p.s; t0 += 8 * p.splits) {
+        float4 part[2][8];
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
-          part[q] = q < p.splits ? ld_shared_cluster_f32(map_to_cta(mine + t * 512, q)) : 0.0f;
-        float acc = part[0];
+        for (int u = 0; u < 2; ++u) {
+          const int t = t0 + 4 * u * p.splits;
 #pragma unroll
-        for (int q = 1; q < 8; ++q) acc += part[q];
-        if (mrow < p.m) {
-          if (OUT_BF16)
-            reinterpret_cast<__nv_bfloat16*>(p.y)[t * p.ldy + mrow] = __float2bfloat16_rn(acc);
-          else
-            reinterpret_cast<float*>(p.y)[t * p.ldy + mrow] = acc;
+          for (int q = 0; q < 8; ++q)
+            part[u][q] = (q < p.splits && t < p.s) ? ld_shared_cluster_v4(map_to_cta(mine + t * 512, q))
+                                                   : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const int t = t0 + 4 * u * p.splits;
+          if (t >= p.s) break;
+          float4 acc = part[u][0];
+#pragma unroll
+          for (int q = 1; q < 8; ++q) {
+            acc.x += part[u][q].x; acc.y += part[u][q].y; acc.z += part[u][q].z; acc.w += part[u][q].w;
+          }
+          if (OUT_BF16) {
+            const __nv_bfloat162 h0 = __floats2bfloat162_rn(acc.x, acc.y), h1 = __floats2bfloat162_rn(acc.z, acc.w);
+            __nv_bfloat16* yp = reinterpret_cast<__nv_bfloat16*>(p.y) + t * p.ldy + m0;
+            if (m0 + 3 < p.m) {
+              *reinterpret_cast<uint2*>(yp) = make_uint2(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
+            } else {
+              if (m0 < p.m) yp[0] = h0.x;
+              if (m0 + 1 < p.m) yp[1] = h0.y;
+              if (m0 + 2 < p.m) yp[2] = h1.x;
+            }
+          } else {
+            float* yp = reinterpret_cast<float*>(p.y) + t * p.ldy + m0;
+            if (m0 + 3 < p.m) {
+              *reinterpret_cast<float4*>(yp) = acc;
+            } else {
+              if (m0 < p.m) yp[0] = acc.x;
+              if (m0 + 1 < p.m) yp[1] = acc.y;
+              if (m0 + 2 < p.m) yp[2] = acc.z;
+            }
+          }
         }
       }
     }
