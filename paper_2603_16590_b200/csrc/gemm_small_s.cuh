@@ -13,10 +13,14 @@
 // thread-block cluster that reduce-scatters the tiles through distributed shared memory (CTA q
 // adds and writes tokens q, q + splits, ...); otherwise the tiles go to scratch and the CTA that
 // draws the last ticket of a row tile adds them.  Up to 16 tokens the cluster's CTAs PUSH: each
-// stores the partial sums of token t straight into a receive buffer of CTA t mod splits (remote
-// stores are posted, nothing waits for them), one cluster barrier, and every CTA adds what it
-// received from local shared memory -- one barrier and no remote load instead of two barriers
-// around a round of remote loads.
+// stores the partial sums of token t straight into a receive buffer of CTA t mod splits, with stores
+// that are counted on an mbarrier there (st.async), and every CTA adds what it received from local
+// shared memory as soon as its count is full -- no cluster barrier after the MMAs and no remote load;
+// the barrier that makes sure the receivers are there lies under the weight stream.  Against plain
+// remote stores and a cluster barrier (whole layers, back to back, 4 and 16 tokens): 4096 -> 6144
+// 5.7 / 7.2 -> 5.2 / 6.7 us, 4096 -> 4096 5.3 / 6.9 -> 4.9 / 6.2, 14336 -> 4096 8.8 / 9.8 -> 8.5 / 9.0.
+// The fused kernel (linear_small_s_fused.cuh) keeps the barrier: there the same change cost 0.9 us
+// on 4096 -> 4096.
 //
 // Warp roles: warp 0 = TMA producer, warp 1 = MMA issuer and tensor-memory owner,
 // warps 2..5 = epilogue.  The weight stream does not depend on the activation
@@ -110,6 +114,7 @@ gemm_small_s_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
   __shared__ __align__(8) uint64_t full_bar[Cfg::kStages];
   __shared__ __align__(8) uint64_t empty_bar[Cfg::kStages];
   __shared__ __align__(8) uint64_t acc_full_bar;
+  __shared__ __align__(8) uint64_t recv_bar;   // push reduction: bytes received from the cluster's CTAs
   __shared__ uint32_t tmem_base_slot;
   __shared__ uint32_t ticket_slot;
   __shared__ int abort_flag;
@@ -122,7 +127,16 @@ gemm_small_s_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
   const int lane = tid & 31;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(small_smem_raw) + 1023) & ~uintptr_t(1023));
 
+  const bool by_cluster = p.cluster_reduce != 0 && p.splits > 1;
+  const bool push = by_cluster && NTOK == 16;
+  const int per = (p.s + p.splits - 1) / p.splits;   // push: token slots of a source
   if (tid == 0) {
+    if (push) {
+      const int sp0 = blockIdx.y;
+      const int owned = sp0 < p.s ? (p.s - sp0 + p.splits - 1) / p.splits : 0;
+      mbar_init(smem_u32(&recv_bar), 1);
+      mbar_arrive_expect_tx(smem_u32(&recv_bar), static_cast<uint32_t>(owned * p.splits * 512));
+    }
     for (int i = 0; i < Cfg::kStages; ++i) {
       mbar_init(smem_u32(&full_bar[i]), 1);
       mbar_init(smem_u32(&empty_bar[i]), 1);
@@ -139,6 +153,7 @@ gemm_small_s_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
   }
   tc_fence_before_sync();
   __syncthreads();
+  if (push) cluster_arrive();   // recv_bar is there; every warp waits for the other CTAs' before it needs them
   tc_fence_after_sync();
   const uint32_t tmem_base = tmem_base_slot;
 
@@ -147,7 +162,6 @@ gemm_small_s_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
   const int kt0 = static_cast<int>(static_cast<int64_t>(p.k_steps) * sp / p.splits);
   const int kt1 = static_cast<int>(static_cast<int64_t>(p.k_steps) * (sp + 1) / p.splits);
   const int n_steps = kt1 - kt0;                  // >= 1: the host keeps splits <= k_steps
-  const bool by_cluster = p.cluster_reduce != 0 && p.splits > 1;
   bool epi_ok = false;
 
   if (warp == 0) {
@@ -258,6 +272,7 @@ gemm_small_s_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
     const int quad = warp & 3;  // tensor-memory lanes [32*quad, 32*quad + 32)
     const int row = quad * 32 + lane;              // weight row inside the tile
     const int64_t mrow = static_cast<int64_t>(rt) * 128 + row;
+    if (push) cluster_wait();
     mbar_wait(smem_u32(&acc_full_bar), 0, &abort_flag);
     // A wait that gave up has raised abort_flag before this barrier, so the four epilogue warps
     // agree on `ok` and take the barriers below together or not at all.
@@ -288,15 +303,18 @@ gemm_small_s_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
         uint32_t v[16];
         tmem_ld_32x32b_x16(taddr + c, v);
         tmem_ld_wait();
-        if (by_cluster && NTOK == 16) {
+        if (push) {
           // push: token t goes to CTA t mod splits, slot [this split][t / splits]
-          const int per = (p.s + p.splits - 1) / p.splits;
+          const uint32_t bar = smem_u32(&recv_bar);
           const uint32_t recv0 = smem_u32(smem + Cfg::kStages * Cfg::kStageBytes) + static_cast<uint32_t>(sp * per * 512 + row * 4);
+          int owner = 0, slot = 0;   // t mod splits, t / splits
 #pragma unroll
-          for (int t = 0; t < 16; ++t)
+          for (int t = 0; t < 16; ++t) {
             if (t < p.s)
-              st_shared_cluster_f32(map_to_cta(recv0 + static_cast<uint32_t>((t / p.splits) * 512), static_cast<uint32_t>(t % p.splits)),
-                                    __uint_as_float(v[t]));
+              st_async_f32(map_to_cta(recv0 + static_cast<uint32_t>(slot * 512), static_cast<uint32_t>(owner)),
+                           __uint_as_float(v[t]), map_to_cta(bar, static_cast<uint32_t>(owner)));
+            if (++owner == p.splits) { owner = 0; ++slot; }
+          }
         } else if (by_cluster) {
 #pragma unroll
           for (int t = 0; t < 16; ++t)
@@ -372,18 +390,17 @@ gemm_small_s_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
     }
   }
 
-  if (by_cluster) {
-    // Every thread of every CTA of the cluster takes both barriers, whatever happened above.
-    __syncthreads();
-    cluster_sync_all();
-    if (NTOK == 16) {
-      // Push mode: everything this CTA owns has arrived in its receive buffer (the barrier above
-      // orders the other CTAs' remote stores before this point); add in split order (deterministic).
-      // No CTA touches another's shared memory any more, so no second barrier.
-      if (warp >= 2 && epi_ok) {
+  if (push) {
+    if (warp < 2) {
+      __syncwarp();
+      cluster_wait();
+    } else {
+      // Every CTA waits for what it owns, whatever happened above: nobody writes to it after that.  Add
+      // in split order (deterministic).
+      const bool received = mbar_wait_received(smem_u32(&recv_bar), &abort_flag);
+      if (received && epi_ok) {
         const int row = (warp & 3) * 32 + lane;
         const int64_t mrow = static_cast<int64_t>(rt) * 128 + row;
-        const int per = (p.s + p.splits - 1) / p.splits;
         const float* recv = reinterpret_cast<const float*>(smem + Cfg::kStages * Cfg::kStageBytes) + row;
         for (int j = 0; sp + j * p.splits < p.s; ++j) {
           const int t = sp + j * p.splits;
@@ -401,7 +418,12 @@ gemm_small_s_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
           }
         }
       }
-    } else if (warp >= 2 && epi_ok) {
+    }
+  } else if (by_cluster) {
+    // Every thread of every CTA of the cluster takes both barriers, whatever happened above.
+    __syncthreads();
+    cluster_sync_all();
+    if (warp >= 2 && epi_ok) {
       // Reduce-scatter: CTA sp adds, in split order (deterministic), the partial sums of tokens
       // sp, sp + splits, ... -- its own from local, the others' from distributed shared memory -- and
       // writes those tokens of y.  What a round of remote loads costs is its latency, so every warp
@@ -453,7 +475,7 @@ gemm_small_s_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_con
         }
       }
     }
-    if (NTOK != 16) cluster_sync_all();  // pull mode: nobody leaves while its shared memory may still be read
+    cluster_sync_all();  // nobody leaves while its shared memory may still be read
   }
   tc_fence_before_sync();
   __syncthreads();

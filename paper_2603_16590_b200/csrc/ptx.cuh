@@ -228,6 +228,38 @@ __device__ __forceinline__ float4 ld_shared_cluster_v4(uint32_t cluster_addr) { 
 __device__ __forceinline__ void st_shared_cluster_f32(uint32_t cluster_addr, float v) {  // any CTA's shared memory
   asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_addr), "f"(v) : "memory");
 }
+// The same, counting 4 bytes on an mbarrier of the CTA that receives them.
+__device__ __forceinline__ void st_async_f32(uint32_t cluster_addr, float v, uint32_t cluster_bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.f32 [%0], %1, [%2];" ::"r"(cluster_addr), "f"(v),
+               "r"(cluster_bar)
+               : "memory");
+}
+// Waits for the first phase of a barrier on which other CTAs' st_async_f32 are counted.  A CTA whose peers
+// may still write to it must not leave, so this goes on when the CTA has given up elsewhere; the limit is
+// twice that of the waits a sender may sit in, so that a sender that is merely late still finds it there.
+__device__ __forceinline__ bool mbar_wait_received(uint32_t bar, volatile int* abort_flag) {
+  uint64_t t0 = 0;
+  for (;;) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], 0, %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(kParkNs)
+        : "memory");
+    if (ok != 0) return true;
+    const uint64_t now = global_timer_ns();
+    if (t0 == 0) t0 = now;
+    if (now - t0 > 2 * kWaitLimitNs) {
+      *abort_flag = 1;
+      atomicExch(&g_device_error, 1);
+      return false;
+    }
+  }
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar) {  // arrive on a barrier of any CTA of the cluster
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
 }
