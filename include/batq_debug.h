@@ -48,11 +48,13 @@ int32_t batq_debug_wide_schedule(int64_t s, int64_t m, int64_t n, int32_t sm_cou
 void batq_debug_force_gemm_kernel(int32_t which);
 
 /* Which activation quantiser later calls use.  0 = automatic (up to 128 tokens the per-block ALU
- * kernel, above that the tensor-core dense-block kernel; the identity transform above 128 tokens
- * and nothing else takes the streaming ALU kernel), 1 = the streaming ALU kernel (Kronecker
- * form), 2 = the tensor-core kernel, 3 = the per-block ALU kernel.  The streaming ALU kernel is
- * built for 4 x 8 factors and the per-block ALU kernel for 4 x 8, 8 x 4 and 16 x 2; a transform
- * of another size takes the tensor-core kernel where the forced one cannot run it. */
+ * kernel or, from 8192 (token, block) items on, the thread-per-item ALU kernel, above that the
+ * tensor-core dense-block kernel; the identity transform above 128 tokens and nothing else takes the
+ * streaming ALU kernel), 1 = the streaming ALU kernel (Kronecker form), 2 = the tensor-core kernel,
+ * 3 = the per-block ALU kernel, 4 = the thread-per-item ALU kernel.  The streaming ALU kernel is
+ * built for 4 x 8 factors, the per-block one for 4 x 8, 8 x 4 and 16 x 2, the thread-per-item one for
+ * 4 x 8 and 8 x 4; a transform of another size takes the tensor-core kernel where the forced one
+ * cannot run it.  batq_quantize_act_mxfp8 takes the tensor-core kernel unless 3 or 4 is forced. */
 void batq_debug_force_quantizer(int32_t which);
 
 /* Number of K splits of the small-s GEMM (clamped to the number of 256-element K steps and to

@@ -1055,9 +1055,6 @@ batq_status launch_gemm(const void* x_codes, const void* x_sf, const batq_weight
   return BATQ_OK;
 }
 
-// Fewer 128-feature tiles than half the SMs.
-bool few_row_tiles(const batq_weight* w) { return (w->m + 127) / 128 * 2 <= w->sm_count; }
-
 // ---- small-s (decode) GEMM: split choice, scratch layout, launch -------------------------------
 std::atomic<int> g_force_splits{0};  // tuning hook: 0 = automatic
 std::atomic<int> g_small_reduce{0};  // tuning hook: 0 = automatic, 1 = always tickets, 2 = cluster whenever splits <= 8
@@ -1229,9 +1226,12 @@ int pick_fused_splits(int64_t m, int64_t n, int sm_count) {
   return best;
 }
 
-// Automatic choice: every CTA of a K split requantises its slice of the activations, which is only
-// hidden behind the weight stream while that is a few items per thread (tokens x K-steps <= 4) and
-// the grid fits the SMs in one wave; measured, the fused kernel then saves about 5 % of a call.
+// Automatic choice: every CTA of a K split requantises its slice of the activations, which only pays
+// while that is next to nothing: one K-step per CTA and up to four tokens (1024 -> 1024: 3.3-3.6 us
+// against 3.9 of the two kernels, 2048 -> 2048 3.6-4.1 against 4.1), or one token and up to four
+// K-steps (4096 -> 6144 and 4096 -> 4096: as quick on the device, one launch less on the host; at two
+// tokens 6.0 / 5.0 against 5.0 / 4.9).  The clusters need room as in cluster_reduce_ok: 288 CTAs of 296
+// slots (3584 -> 4608) took 8.1 us against 4.9.
 bool use_fused_small(const batq_transform* t, const batq_weight* w, int64_t s) {
   const int force_path = g_force_small_path.load(std::memory_order_relaxed);
   if (force_path == 1 || s > kFusedTok) return false;
@@ -1242,7 +1242,7 @@ bool use_fused_small(const batq_transform* t, const batq_weight* w, int64_t s) {
   const int64_t k_steps = (w->n + 255) / 256;
   const int64_t per = (k_steps + sp - 1) / sp;
   const int64_t slots = 2 * static_cast<int64_t>(w->sm_count > 0 ? w->sm_count : 148);
-  return s * per <= 4 && ((w->m + 127) / 128) * sp <= slots;
+  return (per == 1 ? s <= 4 : s == 1 && per <= 4) && ((w->m + 127) / 128) * sp * 10 <= slots * 9;
 }
 
 batq_status launch_linear_fused(const batq_transform* t, const batq_weight* w, const void* x, int64_t s, int64_t ld,
@@ -1403,9 +1403,9 @@ batq_status launch_gemm_w4a8(const void* x_codes8, const void* x_sf, const batq_
   // 7.0 / 11.5 us (4096 -> 6144), 6.1 / 11.2 (4096 -> 4096), 14.4 / 25.5 (4096 -> 28672), 10.7 / 36
   // (14336 -> 4096); at 75 / 96 tokens 11.5 / 12.3 against 11.8 / 11.8 (4096 -> 6144) and 21.9 / 22.6
   // against 22.1 / 22.3 (4096 -> 28672), but 18.0 against 32.8 at 96 and 21.2 against 34.4 at 128 on
-  // 14336 -> 4096: above 80 tokens only large layers with few features.
+  // 14336 -> 4096: above 80 tokens only large layers.
   if (g_force_gemm_kernel.load(std::memory_order_relaxed) == 0 &&
-      (s <= 80 || (s <= kSmallSMax && w->m * w->n >= 40000000 && few_row_tiles(w))))
+      (s <= 80 || (s <= kSmallSMax && w->m * w->n >= 40000000)))
     return launch_gemm_small(x_codes8, x_sf, w, s, y, y_dtype, ldy, nullptr, small_scratch_a8(w, s), stream, dependent, true);
   const bool bf = y_dtype == BATQ_BF16;
   CUtensorMap tmap_a, tmap_y;
@@ -1940,16 +1940,14 @@ batq_status batq_gemm_mxfp4_small_s(const void* x_codes, const void* x_scales_mm
 }
 
 // The whole layer takes the small-s path (ALU quantiser + swapped-operand split-K GEMM) up to 32
-// tokens, up to 64 where the layer is large enough for the weight stream to dominate (>= 40 M weights),
-// and up to 128 where such a layer also has too few features to fill the chip without splitting K.
-// Measured against the one-CTA-per-tile GEMM behind the same quantiser, back to back: 4096 -> 6144 at
-// 32 / 48 / 64 tokens 7.9 / 9.0 / 9.6 us against 10.5 / 9.0 / 8.1; 4096 -> 28672 at 48 / 64 / 75 / 96 /
-// 128 tokens 14.5 / 15.8 / 17.1 / 17.9 / 18.9 against 20.9 / 17.4 / 17.1 / 17.3 / 17.7; 14336 -> 4096 at
-// 75 / 128 tokens 14.0 / 18.0 against 21.1 / 22.7.
+// tokens, and up to 128 where the layer is large enough for the weight stream to dominate (>= 40 M
+// weights).  Measured against the one-CTA-per-tile GEMM behind the same quantiser, back to back:
+// 4096 -> 6144 at 32 / 48 / 64 tokens 7.9 / 9.0 / 9.6 us against 10.5 / 9.0 / 8.1; 4096 -> 28672 at 48 /
+// 64 / 75 / 128 tokens 14.5 / 15.8 / 17.1 / 18.9 against 20.9 / 17.4 / 17.1 / 17.7 (but a layer of 75
+// tokens whose other weights pass through L2 as well is 1.5 us quicker with it: the ring is full of
+// weights before the activations are there); 14336 -> 4096 at 75 / 128 tokens 14.0 / 18.0 against 21.1 / 22.7.
 static bool layer_takes_small_path(const batq_weight* w, int64_t s) {
-  if (s <= 32) return true;
-  if (s > kSmallSMax || w->m * w->n < 40000000) return false;
-  return s <= 64 || few_row_tiles(w);
+  return s <= 32 || (s <= kSmallSMax && w->m * w->n >= 40000000);
 }
 
 size_t batq_linear_workspace_bytes(const batq_weight* w, int64_t s) {

@@ -909,6 +909,26 @@ def test_linear_kernel_launches_reports_the_dispatch(batq):
         batq.batq_debug_force_small_s_path(0)
 
 
+@pytest.mark.parametrize("M,N,S,launches", [(1024, 1024, 4, 1), (1024, 1024, 5, 2), (4096, 4096, 1, 1),
+                                            (4096, 4096, 2, 2), (4608, 3584, 1, 2)])
+def test_fused_decode_dispatch(batq, M, N, S, launches):
+    """One K-step per CTA: up to four tokens; more: one token; never where the clusters of K splits would
+    fill more than 90 % of the CTA slots (4608 features: 36 x 8 of 296).  The result is the oracle's either way."""
+    t = synth.make_transform(N, 3, "baseline")
+    tr = _mk_transform(batq, t)
+    xb, wb = synth.make_activations(S, N, 4), synth.make_weight(M, N, 3)
+    w = batq.batq_prepare_weight(tr, batq.bits_to_cuda_bf16(wb))
+    assert batq.batq_linear_kernel_launches(tr, w, S) == launches
+    y = torch.empty((S, M), dtype=torch.float32, device="cuda")
+    batq.batq_linear_w4a4(tr, w, batq.bits_to_cuda_bf16(xb), y, batq.aligned_workspace(batq.batq_linear_workspace_bytes(w, S)))
+    assert batq.batq_last_device_status() == 0
+    Y, Sabs, _, _ = O.linear_w4a4(xb, wb, t.left, t.right, t.clip_lo, t.clip_hi)
+    got = y.cpu().numpy().astype(np.float64)
+    # as the other whole-layer tests: a flipped activation code moves an output by one grid step of one element
+    assert np.mean(np.abs(got - Y) > 1e-3 * Sabs + 1e-30) <= 1e-3
+    assert np.linalg.norm(got - Y) <= 1e-4 * np.linalg.norm(Sabs)
+
+
 @pytest.mark.parametrize("S,M,N,pinned", [(96, 256, 512, True), (2048, 520, 1024, True), (640, 264, 2048, True),
                                           (1000, 1104, 768, False)])
 def test_linear_host_entry_point_matches_device_entry_point(batq, S, M, N, pinned):
