@@ -1065,14 +1065,15 @@ inline int small_ntok(int64_t s) { return s <= 16 ? 16 : (s <= 32 ? 32 : (s <= 6
 
 // The K splits of a row tile can meet as one thread-block cluster (reduction through distributed
 // shared memory) when there are at most 8 of them and the grid leaves the gang scheduler of
-// clusters some room: at most 90 % of the two-per-SM slots, 80 % above 4 tokens, where the CTAs
-// of the quantiser in front (tokens x blocks / 32 of them, resident while they wait) take room
-// too.  Measured: a fuller grid leaves a few clusters for a second wave, which costs a layer of
-// the decode benchmark about 5 us.
+// clusters some room: at most 80 % of the two-per-SM slots, 90 % for a single token, where the CTAs
+// of the quantiser in front (resident while they wait) take next to none.  Measured, a layer of qkv, o,
+// gate/up and down (14336 -> 4096: 7 splits of 32 row tiles against 8): 34.1 us with 90 % and 33.0
+// with 80 at 2 to 4 tokens, 33.4 / 38.2 with 80 / 90 at 5, 34.3 / 40.6 at 8, 32.7 / 33.3 with 90 / 80 at
+// one token; 72 %: 35.3 at one token, 37.3 at 8.
 bool cluster_reduce_ok(int64_t tiles, int sp, int64_t slots, int64_t s) {
   const int force_reduce = g_small_reduce.load(std::memory_order_relaxed);
   if (sp < 2 || sp > 8 || force_reduce == 1) return false;
-  return force_reduce == 2 || tiles * sp * 10 <= slots * (s > 4 ? 8 : 9);
+  return force_reduce == 2 || tiles * sp * 10 <= slots * (s > 1 ? 8 : 9);
 }
 
 // Number of K splits: the grid is (row tiles) x (splits) CTAs, two resident per SM.  Modelled
