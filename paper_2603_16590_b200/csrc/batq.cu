@@ -389,7 +389,7 @@ bool alu_small_geometry(const batq_transform* t) {
   return t == nullptr || t->gc == 8 || t->gc == 4 || t->gc == 2;
 }
 
-// Per-block ALU version: four lanes per (token, block); fp8: E4M3 codes instead of E2M1.
+// Per-block ALU version: four lanes per (token, block); fp8: E4M3 codes instead of E2M1 (4 x 8 and 8 x 4 factors).
 batq_status launch_quantize_small(const batq_transform* t, const void* x, int64_t s, int64_t n, int64_t ld, void* codes,
                                   void* scales, int32_t layout, float* debug_out, cudaStream_t stream,
                                   uint32_t* zero_words, int32_t n_zero_words, bool fp8) {
@@ -426,10 +426,11 @@ batq_status launch_quantize_small(const batq_transform* t, const void* x, int64_
   const int gc = t != nullptr ? t->gc : 8;
   const bool dbg = debug_out != nullptr;
   cudaError_t e;
-#define BATQ_QS(GC) (fp8   ? cudaLaunchKernelEx(&cfg, quantize_act_small_kernel<false, GC, true>, q) \
-                     : dbg ? cudaLaunchKernelEx(&cfg, quantize_act_small_kernel<true, GC>, q)       \
-                           : cudaLaunchKernelEx(&cfg, quantize_act_small_kernel<false, GC>, q))
-  e = gc == 8 ? BATQ_QS(8) : gc == 4 ? BATQ_QS(4) : BATQ_QS(2);
+#define BATQ_QS(GC) (dbg ? cudaLaunchKernelEx(&cfg, quantize_act_small_kernel<true, GC>, q) \
+                         : cudaLaunchKernelEx(&cfg, quantize_act_small_kernel<false, GC>, q))
+  if (fp8) e = gc == 8 ? cudaLaunchKernelEx(&cfg, quantize_act_small_kernel<false, 8, true>, q)
+                       : cudaLaunchKernelEx(&cfg, quantize_act_small_kernel<false, 4, true>, q);
+  else e = gc == 8 ? BATQ_QS(8) : gc == 4 ? BATQ_QS(4) : BATQ_QS(2);
 #undef BATQ_QS
   if (e != cudaSuccess) { cudaGetLastError(); return BATQ_ERR_CUDA; }
   return BATQ_OK;
@@ -498,14 +499,18 @@ constexpr int64_t kWarpQuantMin = 8192;
 bool warp_quant_geometry(const batq_transform* t) { return t != nullptr && !t->bf16_mid && (t->gc == 8 || t->gc == 4); }
 
 // The MXFP8 quantiser of a layer.  batq_quantize_act_mxfp8, whose bytes a caller may keep and compare,
-// has the tensor-core kernel at every size.
+// has the tensor-core kernel at every size.  With 16 x 2 factors the layer has it too: the ALU kernels'
+// fp32 transform is 6.7e-8 off the exact one (2-norm, N(0,1) activations) with 4 x 8 and 8 x 4 factors,
+// where the tensor cores' is 7.1e-8 off, but 8.0e-8 with 16 x 2.
+bool alu_fp8_geometry(const batq_transform* t) { return t->gc == 8 || t->gc == 4; }
 batq_status launch_quantize_layer_fp8(const batq_transform* t, const void* x, int64_t s, int64_t n, int64_t ld, void* codes,
                                       void* scales, cudaStream_t stream, int sm_count) {
   const int force_q = g_force_quantizer.load(std::memory_order_relaxed);
   const bool small = force_q == 0 && s <= small_quant_limit(t);
-  if (warp_quant_geometry(t) && (force_q == 4 || (small && s * (n / 32) > kWarpQuantMin)))
+  if (!alu_fp8_geometry(t)) return launch_quantize_tc(t, x, s, n, ld, codes, scales, BATQ_SF_MMA, nullptr, stream, sm_count, true);
+  if (force_q == 4 || (small && s * (n / 32) > kWarpQuantMin))
     return launch_quantize_warp(t, x, s, n, ld, codes, scales, BATQ_SF_MMA, stream, sm_count, nullptr, 0, true);
-  if (alu_small_geometry(t) && (force_q == 3 || small))
+  if (force_q == 3 || small)
     return launch_quantize_small(t, x, s, n, ld, codes, scales, BATQ_SF_MMA, nullptr, stream, nullptr, 0, true);
   return launch_quantize_tc(t, x, s, n, ld, codes, scales, BATQ_SF_MMA, nullptr, stream, sm_count, true);
 }
@@ -1682,10 +1687,10 @@ batq_status batq_quantize_act_mxfp8(const batq_transform* t, const void* x_bf16,
   st = device_setup(&dev, &info);
   if (st != BATQ_OK) return st;
   if (t->device != dev) return BATQ_ERR_CUDA;
-  if (g_force_quantizer.load(std::memory_order_relaxed) == 3 && alu_small_geometry(t))   // tests
+  if (g_force_quantizer.load(std::memory_order_relaxed) == 3 && alu_fp8_geometry(t))   // tests
     return launch_quantize_small(t, x_bf16, s, n, ld, codes, scales, scale_layout, nullptr, static_cast<cudaStream_t>(stream),
                                  nullptr, 0, true);
-  if (g_force_quantizer.load(std::memory_order_relaxed) == 4 && warp_quant_geometry(t))
+  if (g_force_quantizer.load(std::memory_order_relaxed) == 4 && alu_fp8_geometry(t))
     return launch_quantize_warp(t, x_bf16, s, n, ld, codes, scales, scale_layout, static_cast<cudaStream_t>(stream),
                                 info->sm_count, nullptr, 0, true);
   return launch_quantize_tc(t, x_bf16, s, n, ld, codes, scales, scale_layout, nullptr,

@@ -92,7 +92,7 @@ def test_w4a8_128_token_tile_of_a_large_layer(batq):
 
 
 @pytest.mark.parametrize("layout", [0, 1])
-@pytest.mark.parametrize("gr,gc", [(4, 8), (8, 4), (16, 2)])
+@pytest.mark.parametrize("gr,gc", [(4, 8), (8, 4)])
 @pytest.mark.parametrize("S,N", [(1, 32), (5, 96), (32, 1056), (33, 256)])
 def test_mxfp8_per_block_quantiser_vs_tensor_cores(batq, S, N, gr, gc, layout):
     """The ALU quantiser's codes and scale bytes against the tensor-core kernel's: fp32 sums in another
@@ -115,6 +115,31 @@ def test_mxfp8_per_block_quantiser_vs_tensor_cores(batq, S, N, gr, gc, layout):
     assert np.array_equal(out[0][1], out[1][1])
     differ = out[0][0] != out[1][0]
     assert differ.mean() <= 1e-3 and np.abs(out[0][0] - out[1][0]).max() <= 1
+
+
+@pytest.mark.parametrize("gr,gc,S", [(16, 2, 8), (16, 2, 32), (1, 32, 32), (4, 8, 129)])
+def test_w4a8_layer_equals_its_two_steps(batq, gr, gc, S):
+    """Where the layer has the tensor-core quantiser (16 x 2 factors, whose ALU sums are further off the
+    exact ones, the dense geometries, and more than 128 tokens) it is batq_quantize_act_mxfp8 followed by
+    batq_gemm_mxfp8_mxfp4, bit for bit.  4 M elements: fp32 sums in another order flip some of them."""
+    N, M = 16384, 64
+    rounds = -(-(1 << 22) // (S * N))
+    t = synth.make_transform(N, 6, "baseline", gr=gr, gc=gc)
+    tr = _mk(batq, t)
+    w = batq.batq_prepare_weight(tr, batq.bits_to_cuda_bf16(synth.make_weight(M, N, 6)))
+    ws = batq.aligned_workspace(batq.batq_linear_w4a8_workspace_bytes(w, S))
+    codes = torch.empty((S, N), dtype=torch.uint8, device="cuda")
+    sf = torch.empty(batq.batq_sf_bytes(S, N, 1), dtype=torch.uint8, device="cuda")
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(6)
+    for _ in range(rounds):
+        x = torch.randn((S, N), generator=gen, device="cuda").bfloat16()
+        y, y2 = (torch.empty((S, M), dtype=torch.float32, device="cuda") for _ in range(2))
+        batq.batq_linear_w4a8(tr, w, x, y, ws)
+        batq.batq_quantize_act_mxfp8(tr, x, codes, sf, 1)
+        batq.batq_gemm_mxfp8_mxfp4(codes, sf, w, S, y2)
+        assert torch.equal(y, y2)
+    assert batq.batq_last_device_status() == 0
 
 
 @pytest.mark.parametrize("layout", [0, 1])
