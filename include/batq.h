@@ -224,10 +224,10 @@ batq_status batq_linear_w4a4(const batq_transform* t, const batq_weight* w, cons
  * memory, [s x n] bf16 dense) to x_stage_dev, runs batq_linear_w4a4, copies the
  * result from y_stage_dev to y_host; returns after everything has drained.
  * The copies run on two streams the library keeps per device; from 512 tokens
- * on the rows go through in up to four chunks, so that with pinned host memory
- * the copy-in of one chunk, the kernels of the one before and the copy-out of
- * the one before that overlap (token rows are independent: the result is that
- * of one call on all rows).  x_stage_dev (s*n*2 bytes) and y_stage_dev
+ * on the rows go through in up to four chunks of more than 128 rows, so that with
+ * pinned host memory the copy-in of one chunk, the kernels of the one before and
+ * the copy-out of the one before that overlap (token rows are independent: the
+ * result is that of one call on all rows, bit for bit).  x_stage_dev (s*n*2 bytes) and y_stage_dev
  * (s*m*{4,2} bytes) are caller-provided device staging buffers; workspace as
  * for batq_linear_w4a4 with s rows. */
 batq_status batq_linear_w4a4_host(const batq_transform* t, const batq_weight* w, const void* x_host,

@@ -2054,15 +2054,13 @@ static batq_status host_enqueue(const batq_transform* t, const batq_weight* w, c
   // Token rows are independent, so a large batch goes through in up to four chunks of rows: the
   // copy-in of chunk i + 1 and the copy-out of chunk i - 1 run on streams of their own beside
   // the kernels of chunk i (PCIe carries both directions at once).  A small batch is one chunk.
-  int64_t rows_per_chunk = s >= 512 ? ((s + kHostChunks - 1) / kHostChunks + 127) / 128 * 128 : s;
-  int n_chunks = static_cast<int>((s + rows_per_chunk - 1) / rows_per_chunk);
-  if (n_chunks > 1) {   // the workspace was sized for s rows at once: every chunk must fit it too
-    const int64_t last = s - (n_chunks - 1) * rows_per_chunk;
-    if (ws_bytes(rows_per_chunk) > workspace_bytes || ws_bytes(last) > workspace_bytes) {
-      rows_per_chunk = s;
-      n_chunks = 1;
-    }
-  }
+  // Every chunk has more than 128 rows, as the whole batch has: up to 128 the layer takes other
+  // quantisers and K splits, whose fp32 sums are in another order.
+  int n_chunks = s >= 512 ? static_cast<int>(std::min<int64_t>(kHostChunks, s / 129)) : 1;
+  const int64_t rows_per_chunk = s / n_chunks;   // the last chunk takes the rest
+  // the workspace was sized for s rows at once: every chunk must fit it too
+  if (n_chunks > 1 && (ws_bytes(rows_per_chunk) > workspace_bytes || ws_bytes(s - (n_chunks - 1) * rows_per_chunk) > workspace_bytes))
+    n_chunks = 1;
   int dev;
   const DeviceInfo* info;
   batq_status st = device_setup(&dev, &info);
@@ -2075,7 +2073,7 @@ static batq_status host_enqueue(const batq_transform* t, const batq_weight* w, c
   bool ok = stream_follows(hp->in, cs);
   for (int c = 0; c < n_chunks && ok && st == BATQ_OK; ++c) {
     const int64_t r0 = c * rows_per_chunk;
-    const int64_t rows = std::min<int64_t>(rows_per_chunk, s - r0);
+    const int64_t rows = c + 1 < n_chunks ? rows_per_chunk : s - r0;
     const uint8_t* xh = static_cast<const uint8_t*>(x_host) + static_cast<size_t>(r0 * w->n) * 2;
     uint8_t* xd = static_cast<uint8_t*>(x_stage_dev) + static_cast<size_t>(r0 * w->n) * 2;
     uint8_t* yd = static_cast<uint8_t*>(y_stage_dev) + static_cast<size_t>(r0 * w->m) * ysz;

@@ -930,7 +930,8 @@ def test_fused_decode_dispatch(batq, M, N, S, launches):
 
 
 @pytest.mark.parametrize("S,M,N,pinned", [(96, 256, 512, True), (2048, 520, 1024, True), (640, 264, 2048, True),
-                                          (1000, 1104, 768, False)])
+                                          (1000, 1104, 768, False), (512, 264, 4096, True), (513, 264, 4096, True),
+                                          (1153, 264, 4096, True)])
 def test_linear_host_entry_point_matches_device_entry_point(batq, S, M, N, pinned):
     """Host buffers in and out.  From 512 tokens on the rows go through in chunks whose copies and
     kernels overlap; token rows are independent, so the result is bit for bit that of one device

@@ -299,11 +299,12 @@ def test_linear_w4a8_with_row_strides_and_bf16_output(batq):
     assert torch.equal(yp[:, :M], y32.bfloat16()) and (yp[:, M:] == 3.0).all()
 
 
-@pytest.mark.parametrize("S", [96, 2048])
-def test_linear_w4a8_host_entry_point_matches_device_entry_point(batq, S):
+@pytest.mark.parametrize("S,N", [(96, 1024), (2048, 1024), (512, 4096), (513, 4096), (520, 4096), (600, 4096), (640, 4096),
+                                 (641, 4096), (1153, 4096)])
+def test_linear_w4a8_host_entry_point_matches_device_entry_point(batq, S, N):
     """Host buffers in and out for the W4A8 layer (row chunks from 512 tokens on): bit for bit the
-    device entry point's result."""
-    M, N = 520, 1024
+    device entry point's result, also where the rows do not divide into chunks of 128."""
+    M = 520
     xb = synth.make_activations(S, N, 31)
     t = synth.make_transform(N, 31, "baseline")
     tr = _mk(batq, t)
