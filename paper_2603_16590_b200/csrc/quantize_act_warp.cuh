@@ -70,8 +70,13 @@ __global__ void __launch_bounds__(kQwThreads, 3) quantize_act_warp_kernel(const 
   const int j = static_cast<int>(blockIdx.x) * 4 + warp;
   const int t0 = static_cast<int>(blockIdx.y) * p.tiles_per_cta;
   const int t1 = min(p.n_tiles, t0 + p.tiles_per_cta);
+  auto clear = [&] {   // by all warps of CTA (0, 0), those of padding blocks too
+    if (blockIdx.x == 0 && blockIdx.y == 0)
+      for (int i = threadIdx.x; i < p.n_zero_words; i += kQwThreads) p.zero_words[i] = 0u;
+  };
   if (j >= p.k) {   // padding blocks of the scale layout: keep them finite
     grid_dependency_wait();
+    clear();
     if (p.sf_layout != 0)
       for (int t = t0; t < t1; ++t) {
         const int64_t row = static_cast<int64_t>(t) * kQwRows + lane;
@@ -103,8 +108,7 @@ __global__ void __launch_bounds__(kQwThreads, 3) quantize_act_warp_kernel(const 
   if (CLIP) { c_lo = __ldg(p.clip_lo + j); c_hi = __ldg(p.clip_hi + j); }
   // x may come from the grid in front, which may also still read the codes, scales and tickets of its own call
   grid_dependency_wait();
-  if (blockIdx.x == 0 && blockIdx.y == 0)
-    for (int i = threadIdx.x; i < p.n_zero_words; i += kQwThreads) p.zero_words[i] = 0u;
+  clear();
   const uint16_t* xj = p.x + static_cast<int64_t>(j) * 32;
   uint4 x[4];
   auto load = [&](int t) {

@@ -893,6 +893,29 @@ def test_linear_calls_back_to_back_share_a_workspace(batq, S):
         assert torch.equal(a, b)
 
 
+@pytest.mark.parametrize("mode", [3, 4], ids=["perblock", "peritem"])
+@pytest.mark.parametrize("N", [32, 96, 128, 160])
+def test_quantiser_clears_every_split_ticket(batq, mode, N):
+    """The quantiser in front of the small-s GEMM sets one word per row tile to zero, whatever the number
+    of blocks (with less than four, some warps of the thread-per-item kernel have none)."""
+    S, M = 5, 128 * 150
+    tr = _mk_transform(batq, synth.make_transform(N, 3, "baseline"))
+    w = batq.batq_weight_import(torch.zeros((M, N // 2), dtype=torch.uint8, device="cuda"),
+                                torch.full((M, N // 32), 127, dtype=torch.uint8, device="cuda"))
+    need = batq.batq_linear_workspace_bytes(w, S)
+    ws = batq.aligned_workspace(need)
+    ws.fill_(0xA5)
+    batq.batq_debug_force_quantizer(mode)
+    try:
+        batq.batq_linear_w4a4(tr, w, batq.bits_to_cuda_bf16(synth.make_activations(S, N, 3)),
+                              torch.empty((S, M), dtype=torch.bfloat16, device="cuda"), ws)
+    finally:
+        batq.batq_debug_force_quantizer(0)
+    assert batq.batq_last_device_status() == 0
+    tickets = ws[need - 1024:need - 1024 + 4 * 150]    # the scratch ends with them, rounded up to 1024 bytes
+    assert (tickets == 0).all()
+
+
 def test_linear_kernel_launches_reports_the_dispatch(batq):
     """1 = the fused kernel (a token or so on a layer whose K slices are short), 2 = quantiser + GEMM."""
     t = synth.make_transform(4096, 3, "baseline")
