@@ -1067,39 +1067,49 @@ constexpr int kMaxSplits = 32;
 
 inline int small_ntok(int64_t s) { return s <= 16 ? 16 : (s <= 32 ? 32 : (s <= 64 ? 64 : 128)); }
 
-
-// The K splits of a row tile can meet as one thread-block cluster (reduction through distributed
-// shared memory) when there are at most 8 of them and the grid leaves the gang scheduler of
-// clusters some room: at most 80 % of the two-per-SM slots, 90 % for a single token, where the CTAs
-// of the quantiser in front (resident while they wait) take next to none.  Measured, a layer of qkv, o,
-// gate/up and down (14336 -> 4096: 7 splits of 32 row tiles against 8): 34.1 us with 90 % and 33.0
-// with 80 at 2 to 4 tokens, 33.4 / 38.2 with 80 / 90 at 5, 34.3 / 40.6 at 8, 32.7 / 33.3 with 90 / 80 at
-// one token; 72 %: 35.3 at one token, 37.3 at 8.
+// The K splits of a row tile can meet as one thread-block cluster (reduction through distributed shared
+// memory) when there are at most 8 of them and the whole grid is resident at once: what is left over for
+// a second wave costs a call 2.5 to 5 us.  Clusters of 2, 3, ... 8 CTAs, two an SM, that ran at once on
+// the 148 SMs of three devices: 148, 88-90, 70, 52-53, 44-45, 36-37 and 33 (the next one more is the
+// second wave); in percent of the CTA slots 100, 89, 95, 88, 89, 85 and 89.  Allowed is some 5 % less,
+// for the CTAs of the quantiser in front, which are resident while they wait; next to none for one token.
+// (One line at 80 % sent 14336 -> 4352, 34 clusters of 7, to scratch and tickets at 2 to 4 tokens: 11.3
+// us against 9.0; with MXFP8 activations 14336 -> 16384 to a single split: 33 against 26 at 8 tokens.)
+constexpr int kClusterFill[9] = {0, 0, 94, 85, 90, 84, 86, 81, 83};   // percent, by splits
 bool cluster_reduce_ok(int64_t tiles, int sp, int64_t slots, int64_t s) {
   const int force_reduce = g_small_reduce.load(std::memory_order_relaxed);
   if (sp < 2 || sp > 8 || force_reduce == 1) return false;
-  return force_reduce == 2 || tiles * sp * 10 <= slots * (s > 1 ? 8 : 9);
+  return force_reduce == 2 || tiles * sp * 100 <= slots * (kClusterFill[sp] + (s > 1 ? 0 : 4));
 }
 
 // Number of K splits: the grid is (row tiles) x (splits) CTAs, two resident per SM.  Modelled
-// time = waves x (K-steps per CTA + fixed cost) + a reduction term that grows with the splits,
-// plus the round trip through scratch and tickets where the cluster reduction does not apply
-// (all in units of one K-step of streaming, about 0.5 us).
-// `cluster_only`: no scratch to fall back to, only splits that meet as a cluster (MXFP8 activations).
-int pick_splits(int64_t m, int64_t n, int64_t s, int sm_count, bool cluster_only = false) {
+// time = waves x (K-steps per CTA + fixed cost) + what the splits cost, plus the round trip through
+// scratch and tickets where the cluster reduction does not apply: 1.5 us (60 row tiles of 14336
+// channels, 4 splits, 4 tokens: 15.5 us against 13.7).  The unit is a K-step of 256 elements, about 0.25 us.
+// Up to 16 tokens, where a call is mostly latencies, the steps of two CTAs on one SM take up to half as
+// long again; above, they overlap, and the reduction is work of its own (1024 -> 16384, 32 tokens, two
+// splits against one: 1.23 times the time), fewer steps' worth with MXFP8 activations, whose steps are
+// longer.  Fitted to all splits of 24 to 50 layer widths, 1024 to 14336 channels, at 14 token counts: the
+// choice is 0.2 to 2 % behind the best split on average, a flat 0.15 a split was 1.6 to 12 % behind.
+// `a8`: MXFP8 activations; their callers hand over no scratch, so the splits meet as a cluster or there is one.
+int pick_splits(int64_t m, int64_t n, int64_t s, int sm_count, bool a8 = false) {
   const int k_steps = static_cast<int>((n + 255) / 256);
   const int force_splits = g_force_splits.load(std::memory_order_relaxed);
-  if (force_splits > 0) return std::min(std::min(force_splits, k_steps), cluster_only ? 8 : kMaxSplits);
+  if (force_splits > 0) return std::min(std::min(force_splits, k_steps), a8 ? 8 : kMaxSplits);
   const int64_t tiles = (m + 127) / 128;
-  const int64_t slots = 2 * static_cast<int64_t>(sm_count > 0 ? sm_count : 148);
+  const int64_t sms = sm_count > 0 ? sm_count : 148, slots = 2 * sms;
+  const double per_split = a8 ? (s <= 16 ? 0.15 : 0.3) : s <= 4 ? 0.15 : s <= 16 ? 0.2 : 0.5;
+  const double any_split = a8 ? (s <= 4 ? 1.5 : s <= 16 ? 2.5 : 3.0) : s <= 16 ? 3.0 : 5.0;
   int best = 1;
   double best_cost = 1e30;
   for (int sp = 1; sp <= std::min(k_steps, kMaxSplits); ++sp) {
     const int64_t waves = (tiles * sp + slots - 1) / slots;
-    double cost = static_cast<double>(waves) * ((k_steps + sp - 1) / sp + 3.0) + 0.15 * sp;
+    const double per_sm = std::min(2.0, static_cast<double>(tiles * sp) / static_cast<double>(sms));
+    const double step = s <= 16 ? 1.0 + 0.5 * std::max(0.0, per_sm - 1.0) : 1.0;
+    double cost = static_cast<double>(waves) * ((k_steps + sp - 1) / sp * step + 3.0) + per_split * sp + (sp > 1 ? any_split : 0.0);
     if (sp > 1 && !cluster_reduce_ok(tiles, sp, slots, s)) {
-      if (cluster_only) continue;
-      cost += 2.0;
+      if (a8) continue;
+      cost += 6.0;
     }
     if (cost < best_cost - 1e-9) { best_cost = cost; best = sp; }
   }

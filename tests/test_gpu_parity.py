@@ -770,6 +770,16 @@ def test_gemm_small_s_many_splits_and_bf16(batq):
     assert np.array_equal(b.astype(np.float32), want)
 
 
+@pytest.mark.parametrize("S,M,N", [(2, 34 * 128, 14336), (4, 66 * 128, 14336), (3, 83 * 128, 14336), (2, 128 * 128, 4096),
+                                   (16, 128 * 128, 14336), (1, 33 * 128, 14336)])
+def test_clusters_that_run_at_once_need_no_scratch(batq, S, M, N):
+    """Grids that fill 81 to 90 % of the two-per-SM CTA slots of 148 SMs with clusters of 7, 4, 3 and 2: the
+    device holds them all at once, so the K splits meet in shared memory and the scratch is the tickets alone."""
+    w = batq.batq_weight_import(torch.zeros((M, N // 2), dtype=torch.uint8, device="cuda"),
+                                torch.full((M, N // 32), 127, dtype=torch.uint8, device="cuda"))
+    assert batq.batq_gemm_small_s_scratch_bytes(w, S) == 1024
+
+
 def test_gemm_small_s_rejects_large_s_and_short_scratch(batq):
     w = batq.batq_prepare_weight(None, batq.bits_to_cuda_bf16(synth.make_weight(128, 256, 1)))
     z = torch.zeros(1 << 16, dtype=torch.uint8, device="cuda")
