@@ -1116,6 +1116,28 @@ int pick_splits(int64_t m, int64_t n, int64_t s, int sm_count, bool a8 = false) 
   return best;
 }
 
+// Whether the swapped-operand GEMM is the quicker one of two for s <= 128 tokens: it streams the weights
+// over the whole chip by splitting K, and pays for that with every token (reduction, a tile of up to 128
+// tokens per CTA), where one CTA per 128-token tile takes all K-steps of its columns and about the same time
+// for any number of tokens.  With up to one row tile of weights an SM, the K-steps of 256 that the splits
+// save an SM count: one for every 5 tokens pays, one for every 9 with MXFP8, whose steps take twice as long.
+// Two CTAs on an SM take as long as their steps one after another, with MXFP8 three quarters of that.
+// Whole layers cold, swapped operands / one CTA per tile: 14336 -> 4096 (saving 40 to 49) 15.0 / 22 us at 75
+// tokens, 17.9 / 22.6 at 128; 4096 -> 12288 (none) 13.9 / 12.1 and 16.3 / 12.2; MXFP8 4096 -> 6144 (10) 11.5 / 12.2
+// at 80 and 13.9 / 12.8 at 128, 14336 -> 10752 (14) 29.3 / 35.7 at 64, 4096 -> 16384 (4) 17.6 / 15.3 at 80.
+// With more row tiles than SMs neither splits, and the two lie within 5 % of one another from 75 tokens
+// on; behind a short GEMM the ring of the swapped-operand kernel is full before the activations are there,
+// which is worth 1 us up to 80 tokens (a layer of 4096 / 14336 channels: 54.5 / 55.4 us at 72, 60.8 / 60.1 at 128).
+bool swapped_operands_pay(const batq_weight* w, int64_t s, bool a8) {
+  if (s <= 48 || g_force_splits.load(std::memory_order_relaxed) > 0) return true;   // forced splits: tests of that kernel
+  const int64_t tiles = (w->m + 127) / 128, sms = w->sm_count > 0 ? w->sm_count : 148;
+  if (tiles > sms) return s <= 80;
+  const int64_t k_steps = (w->n + 255) / 256, sp = pick_splits(w->m, w->n, s, w->sm_count, a8);
+  const int64_t per = (k_steps + sp - 1) / sp;
+  const int64_t spent2 = tiles * sp > sms ? (a8 ? 3 : 4) * per : 2 * per;   // twice the steps of an SM
+  return (2 * k_steps - spent2) * (a8 ? 9 : 5) > 2 * s;
+}
+
 // Scratch of the small-s GEMM: split-K partial tiles, then one ticket word per row tile.
 struct SmallScratch {
   size_t partial_bytes, ticket_bytes;
@@ -1414,14 +1436,8 @@ batq_status launch_gemm_w4a8(const void* x_codes8, const void* x_sf, const batq_
   if (w->device != dev) return BATQ_ERR_CUDA;
   if (!w->has_u4) return BATQ_ERR_UNSUPPORTED;
   // A handful of tokens: bound by streaming the weights, which the swapped-operand kernel does over
-  // the whole chip whatever the number of features, its K splits meeting as clusters.  Whole layer,
-  // back to back, swapped operands against one CTA per tile behind the same quantiser: at 8 tokens
-  // 7.0 / 11.5 us (4096 -> 6144), 6.1 / 11.2 (4096 -> 4096), 14.4 / 25.5 (4096 -> 28672), 10.7 / 36
-  // (14336 -> 4096); at 75 / 96 tokens 11.5 / 12.3 against 11.8 / 11.8 (4096 -> 6144) and 21.9 / 22.6
-  // against 22.1 / 22.3 (4096 -> 28672), but 18.0 against 32.8 at 96 and 21.2 against 34.4 at 128 on
-  // 14336 -> 4096: above 80 tokens only large layers.
-  if (g_force_gemm_kernel.load(std::memory_order_relaxed) == 0 &&
-      (s <= 80 || (s <= kSmallSMax && w->m * w->n >= 40000000)))
+  // the whole chip whatever the number of features, its K splits meeting as clusters.
+  if (g_force_gemm_kernel.load(std::memory_order_relaxed) == 0 && s <= kSmallSMax && swapped_operands_pay(w, s, true))
     return launch_gemm_small(x_codes8, x_sf, w, s, y, y_dtype, ldy, nullptr, small_scratch_a8(w, s), stream, dependent, true);
   const bool bf = y_dtype == BATQ_BF16;
   CUtensorMap tmap_a, tmap_y;
@@ -1957,13 +1973,9 @@ batq_status batq_gemm_mxfp4_small_s(const void* x_codes, const void* x_scales_mm
 
 // The whole layer takes the small-s path (ALU quantiser + swapped-operand split-K GEMM) up to 32
 // tokens, and up to 128 where the layer is large enough for the weight stream to dominate (>= 40 M
-// weights).  Measured against the one-CTA-per-tile GEMM behind the same quantiser, back to back:
-// 4096 -> 6144 at 32 / 48 / 64 tokens 7.9 / 9.0 / 9.6 us against 10.5 / 9.0 / 8.1; 4096 -> 28672 at 48 /
-// 64 / 75 / 128 tokens 14.5 / 15.8 / 17.1 / 18.9 against 20.9 / 17.4 / 17.1 / 17.7 (but a layer of 75
-// tokens whose other weights pass through L2 as well is 1.5 us quicker with it: the ring is full of
-// weights before the activations are there); 14336 -> 4096 at 75 / 128 tokens 14.0 / 18.0 against 21.1 / 22.7.
+// weights) and the swapped operands pay.
 static bool layer_takes_small_path(const batq_weight* w, int64_t s) {
-  return s <= 32 || (s <= kSmallSMax && w->m * w->n >= 40000000);
+  return s <= 32 || (s <= kSmallSMax && w->m * w->n >= 40000000 && swapped_operands_pay(w, s, false));
 }
 
 size_t batq_linear_workspace_bytes(const batq_weight* w, int64_t s) {

@@ -926,6 +926,18 @@ def test_quantiser_clears_every_split_ticket(batq, mode, N):
     assert (tickets == 0).all()
 
 
+@pytest.mark.parametrize("S,M,N,small", [(32, 128, 4096, True), (33, 128, 4096, False), (48, 12288, 4096, True),
+                                         (64, 12288, 4096, False), (128, 12288, 4096, False), (128, 4096, 14336, True),
+                                         (80, 28672, 4096, True), (81, 28672, 4096, False)])
+def test_small_s_path_of_a_layer_while_its_splits_pay(batq, S, M, N, small):
+    """From 49 tokens on a layer takes the swapped-operand GEMM only where the K splits save enough steps; the
+    workspace has room for its tickets then and only then."""
+    w = batq.batq_weight_import(torch.zeros((M, N // 2), dtype=torch.uint8, device="cuda"),
+                                torch.full((M, N // 32), 127, dtype=torch.uint8, device="cuda"))
+    quantised = S * N // 2 + (-(S * N // 2)) % 1024 + batq.batq_sf_bytes(S, N, 1)
+    assert (batq.batq_linear_workspace_bytes(w, S) > quantised) == small
+
+
 def test_linear_kernel_launches_reports_the_dispatch(batq):
     """1 = the fused kernel (a token or so on a layer whose K slices are short), 2 = quantiser + GEMM."""
     t = synth.make_transform(4096, 3, "baseline")

@@ -85,9 +85,13 @@ def test_w4a8_few_tokens_gemm_vs_oracle_same_codes(batq, S, M, N, splits):
     assert np.max(np.abs(got - Y) / (Sabs + 1e-30)) < 1e-5
 
 
-def test_w4a8_128_token_tile_of_a_large_layer(batq):
-    """The 128-token tile, which automatic dispatch keeps for layers of 40 M weights and more."""
-    got, Y, Sabs = _gemm_case(batq, 128, 5008, 8192, 2700)
+@pytest.mark.parametrize("S,M,N", [(48, 264, 1024), (62, 264, 2048), (64, 264, 2048), (65, 264, 4096), (126, 264, 4096),
+                                   (128, 264, 4096), (128, 5008, 8192)])
+def test_w4a8_gemm_on_either_side_of_the_dispatch(batq, S, M, N):
+    """Swapped operands while the K-steps that the splits save are worth the tokens (7 of 8 steps: up to 62
+    tokens; 14 of 16: up to 125; 40 row tiles of 32 steps: the 128-token tile with clusters), one CTA per
+    tile above."""
+    got, Y, Sabs = _gemm_case(batq, S, M, N, 2700)
     assert np.max(np.abs(got - Y) / (Sabs + 1e-30)) < 1e-5
 
 
