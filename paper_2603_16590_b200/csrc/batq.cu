@@ -1099,7 +1099,7 @@ int pick_splits(int64_t m, int64_t n, int64_t s, int sm_count, bool a8 = false) 
   const int64_t tiles = (m + 127) / 128;
   const int64_t sms = sm_count > 0 ? sm_count : 148, slots = 2 * sms;
   const double per_split = a8 ? (s <= 16 ? 0.15 : 0.3) : s <= 4 ? 0.15 : s <= 16 ? 0.2 : 0.5;
-  const double any_split = a8 ? (s <= 4 ? 1.5 : s <= 16 ? 2.5 : 3.0) : s <= 16 ? 3.0 : 5.0;
+  const double any_split = a8 ? (s <= 8 ? 1.5 : s <= 16 ? 2.5 : 3.0) : s <= 16 ? 3.0 : 5.0;
   int best = 1;
   double best_cost = 1e30;
   for (int sp = 1; sp <= std::min(k_steps, kMaxSplits); ++sp) {
@@ -1266,10 +1266,11 @@ int pick_fused_splits(int64_t m, int64_t n, int sm_count) {
 
 // Automatic choice: every CTA of a K split requantises its slice of the activations, which only pays
 // while that is next to nothing: one K-step per CTA and up to four tokens (1024 -> 1024: 3.3-3.6 us
-// against 3.9 of the two kernels, 2048 -> 2048 3.6-4.1 against 4.1), or one token and up to four
-// K-steps (4096 -> 6144 and 4096 -> 4096: as quick on the device, one launch less on the host; at two
-// tokens 6.0 / 5.0 against 5.0 / 4.9).  The clusters need room as in cluster_reduce_ok: 288 CTAs of 296
-// slots (3584 -> 4608) took 8.1 us against 4.9.
+// against 3.9 of the two kernels, 2048 -> 2048 3.6-4.1 against 4.1), two steps and two tokens while no SM has
+// two CTAs (4096 -> 1024 3.8 against 4.2, 4096 -> 2048 4.2 against 4.3, but 4096 -> 4096 5.2 against 4.9), or one
+// token and up to four K-steps (4096 -> 6144 and 4096 -> 4096: as quick on the device, one launch less on
+// the host).  The clusters need room as in cluster_reduce_ok: 288 CTAs of 296 slots (3584 -> 4608) took
+// 8.1 us against 4.9.
 bool use_fused_small(const batq_transform* t, const batq_weight* w, int64_t s) {
   const int force_path = g_force_small_path.load(std::memory_order_relaxed);
   if (force_path == 1 || s > kFusedTok) return false;
@@ -1280,7 +1281,8 @@ bool use_fused_small(const batq_transform* t, const batq_weight* w, int64_t s) {
   const int64_t k_steps = (w->n + 255) / 256;
   const int64_t per = (k_steps + sp - 1) / sp;
   const int64_t slots = 2 * static_cast<int64_t>(w->sm_count > 0 ? w->sm_count : 148);
-  return (per == 1 ? s <= 4 : s == 1 && per <= 4) && ((w->m + 127) / 128) * sp * 10 <= slots * 9;
+  const int64_t ctas = ((w->m + 127) / 128) * sp;
+  return (per == 1 ? s <= 4 : (s == 1 && per <= 4) || (s == 2 && per == 2 && 2 * ctas <= slots)) && ctas * 10 <= slots * 9;
 }
 
 batq_status launch_linear_fused(const batq_transform* t, const batq_weight* w, const void* x, int64_t s, int64_t ld,

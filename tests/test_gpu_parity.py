@@ -955,9 +955,11 @@ def test_linear_kernel_launches_reports_the_dispatch(batq):
 
 
 @pytest.mark.parametrize("M,N,S,launches", [(1024, 1024, 4, 1), (1024, 1024, 5, 2), (4096, 4096, 1, 1),
-                                            (4096, 4096, 2, 2), (4608, 3584, 1, 2)])
+                                            (4096, 4096, 2, 2), (4608, 3584, 1, 2), (1024, 4096, 2, 1), (2304, 4096, 2, 1),
+                                            (2432, 4096, 2, 2), (1024, 4096, 3, 2), (1024, 5120, 2, 2)])
 def test_fused_decode_dispatch(batq, M, N, S, launches):
-    """One K-step per CTA: up to four tokens; more: one token; never where the clusters of K splits would
+    """One K-step per CTA: up to four tokens; two: two tokens while no SM has two CTAs (18 x 8 of 148); more: one
+    token; never where the clusters of K splits would
     fill more than 90 % of the CTA slots (4608 features: 36 x 8 of 296).  The result is the oracle's either way."""
     t = synth.make_transform(N, 3, "baseline")
     tr = _mk_transform(batq, t)
