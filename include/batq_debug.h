@@ -85,6 +85,10 @@ void batq_debug_force_prefill_path(int32_t which);
  * kernel would and returns normally; the next batq_last_device_status reports BATQ_ERR_TIMEOUT
  * once.  The context stays usable. */
 batq_status batq_debug_wait_timeout(int64_t limit_ns, void* stream);
+/* The same with the wait of the decode GEMM for the partial sums that the other CTAs of its cluster
+ * push to it; that one has a limit of its own (twice as long) and goes on where the CTA has given up
+ * elsewhere. */
+batq_status batq_debug_wait_received_timeout(int64_t limit_ns, void* stream);
 
 /* Measurement: the block-scaled FP4 tensor-core rate of this GPU with nothing else in the way.
  * Every CTA (one per SM; pair != 0: every pair of CTAs, tcgen05 cta_group::2) issues `iters`

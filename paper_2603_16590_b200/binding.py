@@ -64,6 +64,7 @@ SIGNATURES = {
     "batq_linear_w4a4_noalloc": (C.c_int, [_P, _P, _P, _I64, _I64, _P, _I32, _I64, _P]),
     "batq_last_device_status": (C.c_int, [_P]),
     "batq_debug_wait_timeout": (C.c_int, [_I64, _P]),
+    "batq_debug_wait_received_timeout": (C.c_int, [_I64, _P]),
     "batq_debug_mma_peak": (C.c_int, [_I32, _I32, _I32, _I32, C.POINTER(C.c_double), _P]),
     "batq_debug_mma_peak_kind": (None, [_I32]),
     "batq_debug_mma_peak_second_width": (None, [_I32]),
@@ -408,6 +409,11 @@ def batq_last_device_status() -> int:
 def batq_debug_wait_timeout(limit_ns: int):
     """Launches the one-warp kernel whose bounded wait runs out after limit_ns."""
     _check(load().batq_debug_wait_timeout(limit_ns, _stream()), "batq_debug_wait_timeout")
+
+
+def batq_debug_wait_received_timeout(limit_ns: int):
+    """The same with the wait for partial sums from other CTAs of a cluster."""
+    _check(load().batq_debug_wait_received_timeout(limit_ns, _stream()), "batq_debug_wait_received_timeout")
 
 
 def batq_debug_mma_peak(pair: bool, bn: int, iters: int, sf_copies: bool = False) -> float:

@@ -2210,13 +2210,15 @@ void batq_debug_force_small_s_path(int32_t which) { g_force_small_path.store(whi
 void batq_debug_force_small_s_reduce(int32_t which) { g_small_reduce.store(which, std::memory_order_relaxed); }
 void batq_debug_force_prefill_path(int32_t which) { g_force_prefill_path.store(which, std::memory_order_relaxed); }
 
-batq_status batq_debug_wait_timeout(int64_t limit_ns, void* stream) {
+static batq_status launch_wait_timeout(int64_t limit_ns, bool received, void* stream) {
   batq_status st = device_setup(nullptr, nullptr);
   if (st != BATQ_OK) return st;
   const uint64_t lim = static_cast<uint64_t>(std::min<int64_t>(std::max<int64_t>(limit_ns, 1000), 10000000));
-  wait_timeout_kernel<<<1, 32, 0, static_cast<cudaStream_t>(stream)>>>(lim);
+  wait_timeout_kernel<<<1, 32, 0, static_cast<cudaStream_t>(stream)>>>(lim, received);
   return cudaGetLastError() == cudaSuccess ? BATQ_OK : BATQ_ERR_CUDA;
 }
+batq_status batq_debug_wait_timeout(int64_t limit_ns, void* stream) { return launch_wait_timeout(limit_ns, false, stream); }
+batq_status batq_debug_wait_received_timeout(int64_t limit_ns, void* stream) { return launch_wait_timeout(limit_ns, true, stream); }
 
 std::atomic<int> g_peak_load_stages{4};
 std::atomic<int> g_peak_load_sharing{1};

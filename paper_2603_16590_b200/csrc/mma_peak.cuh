@@ -332,7 +332,8 @@ mma_peak_kernel(const __grid_constant__ CUtensorMap tmap_w, const PeakParams p) 
 
 // One warp waits on a barrier nothing signals; the bounded wait gives up after limit_ns, records
 // the time-out for the host and the kernel returns normally.
-__global__ void wait_timeout_kernel(uint64_t limit_ns) {
+// received: with the wait for bytes from other CTAs instead.
+__global__ void wait_timeout_kernel(uint64_t limit_ns, bool received) {
   __shared__ __align__(8) uint64_t bar;
   __shared__ int abort_flag;
   if (threadIdx.x == 0) {
@@ -341,7 +342,10 @@ __global__ void wait_timeout_kernel(uint64_t limit_ns) {
     mbar_fence_init();
   }
   __syncthreads();
-  mbar_wait(smem_u32(&bar), 0, &abort_flag, limit_ns);
+  if (received)
+    mbar_wait_received(smem_u32(&bar), &abort_flag, limit_ns);
+  else
+    mbar_wait(smem_u32(&bar), 0, &abort_flag, limit_ns);
 }
 
 }  // namespace batq

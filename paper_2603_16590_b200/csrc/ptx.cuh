@@ -225,10 +225,7 @@ __device__ __forceinline__ float4 ld_shared_cluster_v4(uint32_t cluster_addr) { 
   asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(cluster_addr) : "memory");
   return v;
 }
-__device__ __forceinline__ void st_shared_cluster_f32(uint32_t cluster_addr, float v) {  // any CTA's shared memory
-  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_addr), "f"(v) : "memory");
-}
-// The same, counting 4 bytes on an mbarrier of the CTA that receives them.
+// Stores to the shared memory of any CTA of the cluster, counting 4 bytes on an mbarrier of that CTA.
 __device__ __forceinline__ void st_async_f32(uint32_t cluster_addr, float v, uint32_t cluster_bar) {
   asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.f32 [%0], %1, [%2];" ::"r"(cluster_addr), "f"(v),
                "r"(cluster_bar)
@@ -237,7 +234,8 @@ __device__ __forceinline__ void st_async_f32(uint32_t cluster_addr, float v, uin
 // Waits for the first phase of a barrier on which other CTAs' st_async_f32 are counted.  A CTA whose peers
 // may still write to it must not leave, so this goes on when the CTA has given up elsewhere; the limit is
 // twice that of the waits a sender may sit in, so that a sender that is merely late still finds it there.
-__device__ __forceinline__ bool mbar_wait_received(uint32_t bar, volatile int* abort_flag) {
+__device__ __forceinline__ bool mbar_wait_received(uint32_t bar, volatile int* abort_flag,
+                                                   uint64_t limit_ns = 2 * kWaitLimitNs) {
   uint64_t t0 = 0;
   for (;;) {
     uint32_t ok;
@@ -251,7 +249,7 @@ __device__ __forceinline__ bool mbar_wait_received(uint32_t bar, volatile int* a
     if (ok != 0) return true;
     const uint64_t now = global_timer_ns();
     if (t0 == 0) t0 = now;
-    if (now - t0 > 2 * kWaitLimitNs) {
+    if (now - t0 > limit_ns) {
       *abort_flag = 1;
       atomicExch(&g_device_error, 1);
       return false;

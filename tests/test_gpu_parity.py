@@ -236,11 +236,12 @@ def test_transform_output_on_exact_ties(batq, mode, layout):
     assert np.array_equal(gc[nz], oc[nz])
 
 
-def test_bounded_wait_runs_out_and_is_reported_once(batq):
+@pytest.mark.parametrize("wait,S", [("batq_debug_wait_timeout", 300), ("batq_debug_wait_received_timeout", 6)])
+def test_bounded_wait_runs_out_and_is_reported_once(batq, wait, S):
     """Failure detection without a fault: one warp waits 1 ms on a barrier nothing signals; the wait
     gives up, the kernel returns, the host reads BATQ_ERR_TIMEOUT exactly once, and the layer that
-    ran before gives the same bits afterwards."""
-    S, M, N = 300, 264, 1024
+    ran before gives the same bits afterwards (6 tokens: the GEMM whose CTAs wait for one another's sums)."""
+    M, N = 264, 1024
     t = synth.make_transform(N, 21, "baseline")
     tr = _mk_transform(batq, t)
     w = batq.batq_prepare_weight(tr, batq.bits_to_cuda_bf16(synth.make_weight(M, N, 21)))
@@ -249,7 +250,7 @@ def test_bounded_wait_runs_out_and_is_reported_once(batq):
     y0 = torch.empty((S, M), dtype=torch.float32, device="cuda")
     batq.batq_linear_w4a4(tr, w, x, y0, ws)
     assert batq.batq_last_device_status() == 0
-    batq.batq_debug_wait_timeout(1_000_000)
+    getattr(batq, wait)(1_000_000)
     assert batq.batq_last_device_status() == 8       # BATQ_ERR_TIMEOUT
     assert batq.batq_last_device_status() == 0       # the record was cleared by the query
     y1 = torch.empty((S, M), dtype=torch.float32, device="cuda")
