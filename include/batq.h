@@ -182,6 +182,12 @@ batq_status batq_gemm_mxfp8_mxfp4(const void* x_codes8, const void* x_scales_mma
 
 /* The whole W4A8 layer: transform + clip + MXFP8 quantisation of X into the workspace (Eq. 1-4,
  * Sec. 2), then batq_gemm_mxfp8_mxfp4, launched as a programmatic dependent of the quantiser.
+ * Above 128 tokens (64 with 8 x 4 factors, and at any number with the other sizes) the codes are those of
+ * batq_quantize_act_mxfp8.  Below, 4 x 8 and 8 x 4 transforms run on the ALUs, whose fp32 sums are in
+ * another order (6.7e-8 off the exact transform, the tensor cores' 7.1e-8): a few codes in a million,
+ * next to a rounding boundary, are the neighbouring one.  The same holds for the order of the GEMM's
+ * fp32 sums, so the last bits of a row may depend on how many rows come with it, as in
+ * batq_linear_w4a4.  Activations are finite; a block with an infinity or NaN has unspecified codes.
  *   t          transform (required, as for batq_quantize_act_mxfp8).
  *   workspace  dev, at least batq_linear_w4a8_workspace_bytes(w, s) bytes, 1024-byte aligned.
  * Errors as batq_linear_w4a4, plus UNSUPPORTED for n % 128 != 0. */
@@ -205,10 +211,10 @@ batq_status batq_gemm_mxfp4_small_s(const void* x_codes, const void* x_scales_mm
                                     size_t scratch_bytes, void* stream);
 
 /* The whole layer, stages 1+2+3: quantise X into the workspace, then the GEMM.  Up to 32
- * tokens (up to 128 on layers of at least 40 M weights) take the small-s GEMM, launched so that
- * its weight stream overlaps the quantiser; the smallest cases take a single kernel that
- * quantises the activations inside the GEMM (no workspace traffic at all).  In every other case
- * the GEMM is launched as a programmatic dependent of the quantiser as well.
+ * tokens (up to 128 on layers of at least 40 M weights where its K splits pay) take the small-s
+ * GEMM, launched so that its weight stream overlaps the quantiser; the smallest cases take a single
+ * kernel that quantises the activations inside the GEMM (no workspace traffic at all).  In every
+ * other case the GEMM is launched as a programmatic dependent of the quantiser as well.
  *   workspace  dev, at least batq_linear_workspace_bytes(w, s) bytes, 1024-byte
  *              aligned; overwritten by every call (calls sharing a workspace
  *              must be ordered on one stream). */

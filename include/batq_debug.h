@@ -42,34 +42,39 @@ int32_t batq_debug_wide_schedule(int64_t s, int64_t m, int64_t n, int32_t sm_cou
 /* Which prefill GEMM kernel later calls use.  0 = automatic (CTA pairs sharing a 256-token tile
  * for s > 128 -- with tiles of up to 256 features and two accumulators, or tiles of up to 448
  * features and one, whichever the cost model expects to finish first --, one CTA per 128-token
- * tile otherwise), 1 = always one CTA per tile, 2 = always CTA pairs with two accumulators,
+ * tile otherwise; batq_gemm_mxfp8_mxfp4 takes the swapped-operand kernel up to 48 tokens, and up to 128
+ * where its K splits pay), 1 = always one CTA per tile, 2 = always CTA pairs with two accumulators,
  * 3 = always CTA pairs with wide tiles (batq_debug_force_tile_width then takes any multiple of 64
  * up to 448 and makes every column that wide). */
 void batq_debug_force_gemm_kernel(int32_t which);
 
 /* Which activation quantiser later calls use.  0 = automatic (up to 128 tokens the per-block ALU
- * kernel or, from 8192 (token, block) items on, the thread-per-item ALU kernel, above that the
+ * kernel or, above 8192 (token, block) items, the thread-per-item ALU kernel, above 128 the
  * tensor-core dense-block kernel; the identity transform above 128 tokens and nothing else takes the
  * streaming ALU kernel), 1 = the streaming ALU kernel (Kronecker form), 2 = the tensor-core kernel,
  * 3 = the per-block ALU kernel, 4 = the thread-per-item ALU kernel.  The streaming ALU kernel is
- * built for 4 x 8 factors, the per-block one for 4 x 8, 8 x 4 and 16 x 2, the thread-per-item one for
- * 4 x 8 and 8 x 4; a transform of another size takes the tensor-core kernel where the forced one
- * cannot run it.  batq_quantize_act_mxfp8 takes the tensor-core kernel unless 3 or 4 is forced. */
+ * built for 4 x 8 factors, the per-block one for 4 x 8, 8 x 4 and, with MXFP4 codes, 16 x 2, the
+ * thread-per-item one for 4 x 8 and 8 x 4; a transform of another size takes the tensor-core kernel where
+ * the forced one cannot run it.  batq_quantize_act_mxfp8 takes the tensor-core kernel unless 3 or 4 is
+ * forced. */
 void batq_debug_force_quantizer(int32_t which);
 
 /* Number of K splits of the small-s GEMM (clamped to the number of 256-element K steps and to
- * 32); 0 restores the automatic choice.  Scratch sizes follow it. */
+ * 32, with MXFP8 activations to 8); 0 restores the automatic choice.  Scratch sizes follow it, and up to
+ * 128 tokens layers for which that GEMM is considered take it. */
 void batq_debug_force_small_s_splits(int32_t splits);
 
 /* How the small-s GEMM adds the partial tiles of its K splits.  0 = automatic (through a
  * thread-block cluster's shared memory where the grid leaves room for clusters, else through
  * scratch and tickets), 1 = always scratch and tickets, 2 = the cluster whenever there are at
- * most 8 splits. */
+ * most 8 splits.  With MXFP8 activations there is no scratch: 1 leaves one split, unless splits are
+ * forced, which then meet as a cluster. */
 void batq_debug_force_small_s_reduce(int32_t which);
 
 /* How batq_linear_w4a4 runs a handful of tokens.  0 = automatic (one fused kernel that quantises
- * the activations inside the GEMM where that is the faster one -- tokens x K-steps per CTA <= 4
- * and a grid of one wave --, else the quantiser kernel followed by the small-s GEMM), 1 = always
+ * the activations inside the GEMM where that is the faster one -- one K-step per CTA and up to four
+ * tokens, two and two while no SM has two CTAs, or one token and up to four, on at most 90 % of the CTA
+ * slots --, else the quantiser kernel followed by the small-s GEMM), 1 = always
  * the two kernels, 2 = the fused kernel up to 16 tokens.  The fused kernel needs n <= 16384;
  * other shapes take the two kernels. */
 void batq_debug_force_small_s_path(int32_t which);

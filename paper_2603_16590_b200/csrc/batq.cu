@@ -324,7 +324,7 @@ batq_status check_x(const void* x, int64_t s, int64_t n, int64_t ld) {
 }
 
 constexpr int64_t kSmallSMax = 128;       // the swapped-operand split-K GEMM takes up to this many tokens
-constexpr int64_t kSmallQuantAuto = 128;  // per-block ALU quantiser up to here, tensor cores above (4.0 us against 1.7-3.0 us back to back at n = 4096)
+constexpr int64_t kSmallQuantAuto = 128;  // ALU quantisers up to here, tensor cores above (4.0 us against 1.7-3.0 us back to back at n = 4096)
 std::atomic<int> g_force_quantizer{0};  // tuning hook: 0 = automatic, 1 = ALU (Kronecker form, streaming), 2 = tensor cores (dense form), 3 = ALU per block, 4 = ALU, thread per item
 
 // Tensor-core version: 128-token x 4-block units.
@@ -490,11 +490,12 @@ int64_t small_quant_limit(const batq_transform* t) {
   return t->gc == 4 ? 64 : t->gc == 2 ? 32 : 0;
 }
 
-// (token, block) items from which the thread-per-item kernel takes over from the per-block one (2.1
-// against 2.4 us at 32 x 4096 = 4096 items, 3.1 against 2.6 at 9600, 8.0 against 4.2 at 57344).  Both
-// give the same codes; the tensor cores' fp32 sums round in another order (6.6e-8 and 8.1e-8 off the
-// exact ones), so above the limit everything stays with them although this kernel would be the quicker
-// one up to some 50000 items (200 x 4096: 3.2 against 4.4 us).
+// (token, block) items above which the thread-per-item kernel takes over from the per-block one (per
+// block / per item: 2.1 / 2.4 us at 32 x 4096 = 4096 items, 3.1 / 2.6 at 9600, 8.0 / 4.2 at 57344).  Both
+// give the same codes; the tensor cores' fp32 sums round in another order (with one channel in a hundred
+// x 50, 6.6e-8 off the exact ones on the ALUs and 8.1e-8 on the tensor cores), so above 128 tokens everything
+// stays with them although this kernel would be the quicker one up to some 50000 items (200 x 4096: 3.2
+// against 4.4 us).
 constexpr int64_t kWarpQuantMin = 8192;
 bool warp_quant_geometry(const batq_transform* t) { return t != nullptr && !t->bf16_mid && (t->gc == 8 || t->gc == 4); }
 
@@ -1075,16 +1076,18 @@ inline int small_ntok(int64_t s) { return s <= 16 ? 16 : (s <= 32 ? 32 : (s <= 6
 // for the CTAs of the quantiser in front, which are resident while they wait; next to none for one token.
 // (One line at 80 % sent 14336 -> 4352, 34 clusters of 7, to scratch and tickets at 2 to 4 tokens: 11.3
 // us against 9.0; with MXFP8 activations 14336 -> 16384 to a single split: 33 against 26 at 8 tokens.)
-constexpr int kClusterFill[9] = {0, 0, 94, 85, 90, 84, 86, 81, 83};   // percent, by splits
+constexpr int kClusterFill[9] = {0, 0, 94, 85, 90, 84, 86, 81, 83};      // percent, by splits
+constexpr int kClusterFillOne[9] = {0, 0, 98, 90, 93, 88, 90, 84, 87};   // one token
 bool cluster_reduce_ok(int64_t tiles, int sp, int64_t slots, int64_t s) {
   const int force_reduce = g_small_reduce.load(std::memory_order_relaxed);
   if (sp < 2 || sp > 8 || force_reduce == 1) return false;
-  return force_reduce == 2 || tiles * sp * 100 <= slots * (kClusterFill[sp] + (s > 1 ? 0 : 4));
+  return force_reduce == 2 || tiles * sp * 100 <= slots * (s > 1 ? kClusterFill : kClusterFillOne)[sp];
 }
 
-// Number of K splits: the grid is (row tiles) x (splits) CTAs, two resident per SM.  Modelled
-// time = waves x (K-steps per CTA + fixed cost) + what the splits cost, plus the round trip through
-// scratch and tickets where the cluster reduction does not apply: 1.5 us (60 row tiles of 14336
+// Number of K splits: the grid is (row tiles) x (splits) CTAs, two resident per SM, all at once: in a second
+// wave no split was ever the quicker choice (10624 -> 39680, 310 row tiles, one token: 45.7 us unsplit, 48.6 and
+// 49.2 with 2 and 3 splits).  Modelled time = K-steps per CTA + what the splits cost, plus the round trip
+// through scratch and tickets where the cluster reduction does not apply: 1.5 us (60 row tiles of 14336
 // channels, 4 splits, 4 tokens: 15.5 us against 13.7).  The unit is a K-step of 256 elements, about 0.25 us.
 // Up to 16 tokens, where a call is mostly latencies, the steps of two CTAs on one SM take up to half as
 // long again; above, they overlap, and the reduction is work of its own (1024 -> 16384, 32 tokens, two
@@ -1102,11 +1105,10 @@ int pick_splits(int64_t m, int64_t n, int64_t s, int sm_count, bool a8 = false) 
   const double any_split = a8 ? (s <= 8 ? 1.5 : s <= 16 ? 2.5 : 3.0) : s <= 16 ? 3.0 : 5.0;
   int best = 1;
   double best_cost = 1e30;
-  for (int sp = 1; sp <= std::min(k_steps, kMaxSplits); ++sp) {
-    const int64_t waves = (tiles * sp + slots - 1) / slots;
+  for (int sp = 1; sp <= std::min(k_steps, kMaxSplits) && (sp == 1 || tiles * sp <= slots); ++sp) {
     const double per_sm = std::min(2.0, static_cast<double>(tiles * sp) / static_cast<double>(sms));
     const double step = s <= 16 ? 1.0 + 0.5 * std::max(0.0, per_sm - 1.0) : 1.0;
-    double cost = static_cast<double>(waves) * ((k_steps + sp - 1) / sp * step + 3.0) + per_split * sp + (sp > 1 ? any_split : 0.0);
+    double cost = (k_steps + sp - 1) / sp * step + per_split * sp + (sp > 1 ? any_split : 0.0);
     if (sp > 1 && !cluster_reduce_ok(tiles, sp, slots, s)) {
       if (a8) continue;
       cost += 6.0;
@@ -1705,7 +1707,7 @@ batq_status batq_quantize_act_mxfp8(const batq_transform* t, const void* x_bf16,
   if (st != BATQ_OK) return st;
   if (t == nullptr) return BATQ_ERR_NULL;
   if (t->n != n) return BATQ_ERR_SHAPE;
-  if (t->bf16_mid) return BATQ_ERR_UNSUPPORTED;   // the 8-bit quantiser has the dense form only
+  if (t->bf16_mid) return BATQ_ERR_UNSUPPORTED;   // the bf16 intermediates are of the factored form, this is the dense one
   if (scale_layout != BATQ_SF_ROWMAJOR && scale_layout != BATQ_SF_MMA) return BATQ_ERR_UNSUPPORTED;
   if (s == 0) return BATQ_OK;
   if (codes == nullptr || scales == nullptr) return BATQ_ERR_NULL;

@@ -11,7 +11,8 @@ from tests.helpers import (code_mismatch_report, fp32_transform_bound, near_roun
 pytestmark = pytest.mark.gpu
 
 # A-priori bounds on the fp32 transform error, relative to sum_e |x_e| |P_ef| of the block, per kernel
-# (quantiser mode: 1 = streaming ALU, 2 = tensor cores, 3 = per-block ALU).
+# (quantiser mode: 1 = streaming ALU, 2 = tensor cores, 3 = per-block ALU, 4 = thread-per-item ALU, which has no
+# fp32 output of its own: the streaming kernel, same fused multiply-adds in the same order, gives its values).
 #   ALU kernels (Kronecker form, fused multiply-adds): an 8-term chain for V R and a 4-term chain for
 #   L^T (V R), each step 2^-24: (gc + gr) * 2^-24 to first order; with margin (gr + gc + 3) * 2^-24.
 #   Tensor-core kernel (dense form): P rounded to fp32 (2^-24), three-term bf16 split (exact),
@@ -19,11 +20,11 @@ pytestmark = pytest.mark.gpu
 #   additions may truncate (2^-23 each; only the two high-term MMAs matter): about 10 * 2^-24; the
 #   same 15 * 2^-24 is asserted.
 # Every end-to-end test prints the largest observed |v^ - V| / (2^-24 * sum|x||P|) next to it.
-FP32_REL_ULPS = {1: 15.0, 2: 15.0, 3: 15.0}
+FP32_REL_ULPS = {1: 15.0, 2: 15.0, 3: 15.0, 4: 15.0}
 FP32_REL = 15 * 2.0 ** -24
 
 
-@pytest.fixture(params=[1, 2, 3], ids=["alu", "tensorcore", "perblock"])
+@pytest.fixture(params=[1, 2, 3, 4], ids=["alu", "tensorcore", "perblock", "peritem"])
 def qmode(request, batq):
     """Runs a test once per activation-quantiser implementation."""
     batq.batq_debug_force_quantizer(request.param)
@@ -125,7 +126,7 @@ def test_identity_transform_is_bit_exact_plain_mxfp4(batq, S, N):
     assert np.array_equal(gs, os_) and np.array_equal(gc, oc)
     # identity *factors* through either transform kernel give the same bits
     t = synth.make_transform(N, 1, identity=True, clip=False)
-    for mode in (1, 2, 3):
+    for mode in (1, 2, 3, 4):
         batq.batq_debug_force_quantizer(mode)
         try:
             gc2, gs2 = _gpu_quantize(batq, _mk_transform(batq, t), xb)
@@ -164,10 +165,10 @@ def _special_rows(N):
 
 
 @pytest.mark.parametrize("layout", [0, 1], ids=["rowmajor", "mma"])
-@pytest.mark.parametrize("mode", [1, 2, 3], ids=["alu", "tensorcore", "perblock"])
+@pytest.mark.parametrize("mode", [1, 2, 3, 4], ids=["alu", "tensorcore", "perblock", "peritem"])
 def test_every_quantiser_on_special_values_with_identity_factors(batq, mode, layout):
     """Zero blocks, signed zeros, ties at every threshold, saturation at +-7, 2^+-100 and a
-    subnormal block through each of the three quantiser kernels (identity factors, no clip, so the
+    subnormal block through each of the four quantiser kernels (identity factors, no clip, so the
     transform is exact and the result must be the plain MXFP4 of X; a zero's sign bit alone is free:
     a sum of products with the identity's zeros gives +0)."""
     N = 256
@@ -194,7 +195,7 @@ def test_every_quantiser_on_special_values_with_identity_factors(batq, mode, lay
 
 
 @pytest.mark.parametrize("layout", [0, 1], ids=["rowmajor", "mma"])
-@pytest.mark.parametrize("mode", [1, 2, 3], ids=["alu", "tensorcore", "perblock"])
+@pytest.mark.parametrize("mode", [1, 2, 3, 4], ids=["alu", "tensorcore", "perblock", "peritem"])
 def test_transform_output_on_exact_ties(batq, mode, layout):
     """A transform with power-of-two entries whose outputs land exactly on rounding boundaries:
     out[r][c] = v[r][c] + v[r][c-1] / 2 (right factor I + shift / 2, left factor I).  Every product
@@ -772,13 +773,14 @@ def test_gemm_small_s_many_splits_and_bf16(batq):
 
 
 @pytest.mark.parametrize("S,M,N", [(2, 34 * 128, 14336), (4, 66 * 128, 14336), (3, 83 * 128, 14336), (2, 128 * 128, 4096),
-                                   (16, 128 * 128, 14336), (1, 33 * 128, 14336)])
+                                   (16, 128 * 128, 14336), (1, 33 * 128, 14336), (1, 88 * 128, 14336), (1, 310 * 128, 10624)])
 def test_clusters_that_run_at_once_need_no_scratch(batq, S, M, N):
     """Grids that fill 81 to 90 % of the two-per-SM CTA slots of 148 SMs with clusters of 7, 4, 3 and 2: the
-    device holds them all at once, so the K splits meet in shared memory and the scratch is the tickets alone."""
+    device holds them all at once, so the K splits meet in shared memory and the scratch is the tickets alone.
+    More row tiles than slots: no splits at all."""
     w = batq.batq_weight_import(torch.zeros((M, N // 2), dtype=torch.uint8, device="cuda"),
                                 torch.full((M, N // 32), 127, dtype=torch.uint8, device="cuda"))
-    assert batq.batq_gemm_small_s_scratch_bytes(w, S) == 1024
+    assert batq.batq_gemm_small_s_scratch_bytes(w, S) == (4 * M // 128 + 1023) // 1024 * 1024
 
 
 def test_gemm_small_s_rejects_large_s_and_short_scratch(batq):
@@ -799,11 +801,11 @@ def test_gemm_small_s_rejects_large_s_and_short_scratch(batq):
                                             (1, 4096, 4096, "baseline"), (16, 6144, 4096, "paper"),
                                             (64, 520, 1024, "baseline"), (65, 520, 1024, "baseline"),
                                             (100, 1032, 3584, "paper"), (128, 4096, 4096, "baseline"),
-                                            (100, 10240, 4096, "baseline"),   # 65..128 tokens on a large layer: small-s path
+                                            (100, 10240, 4096, "baseline"),   # a wide layer of 42 M weights: one CTA per tile
                                             (129, 520, 1024, "baseline"),
                                             (520, 1032, 1024, "baseline")])
 def test_linear_w4a4_vs_oracle(batq, qmode, S, M, N, geometry):
-    # automatic kernel choice: the small-s GEMM up to 64 tokens, one CTA per tile up to 128, CTA pairs above
+    # automatic kernel choice: the small-s GEMM up to 32 tokens, one CTA per tile up to 128, CTA pairs above
     xb = synth.make_activations(S, N, synth.BASE_SEED)
     wb = synth.make_weight(M, N, synth.BASE_SEED)
     t = synth.make_transform(N, synth.BASE_SEED, geometry)
@@ -939,6 +941,50 @@ def test_small_s_path_of_a_layer_while_its_splits_pay(batq, S, M, N, small):
     assert (batq.batq_linear_workspace_bytes(w, S) > quantised) == small
 
 
+@pytest.mark.parametrize("S,M,N,splits", [(75, 264, 4096, 0), (75, 4096, 14336, 0), (100, 320, 131072, 0), (17, 264, 16384, 16)])
+def test_layer_behind_the_thread_per_item_quantiser(batq, S, M, N, splits):
+    """More than 8192 (token, block) items, the layer's own choice of kernels: in front of one CTA per tile, of
+    clusters and of tickets (32 and 16 splits), which the quantiser clears.  Replayed in a graph on one
+    workspace that held garbage; bit for bit the two steps called one by one."""
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(S)
+    t = synth.make_transform(N, 3, "baseline")
+    tr = _mk_transform(batq, t)
+    w = batq.batq_weight_import(torch.randint(0, 256, (M, N // 2), generator=gen, dtype=torch.uint8, device="cuda"),
+                                torch.randint(118, 128, (M, N // 32), generator=gen, dtype=torch.uint8, device="cuda"))
+    x = torch.randn((S, N), generator=gen, device="cuda").bfloat16()
+    batq.batq_debug_force_small_s_splits(splits)
+    try:
+        small = S <= 32 or M * N >= 40_000_000
+        ws = batq.aligned_workspace(batq.batq_linear_workspace_bytes(w, S))
+        ws.fill_(0xA5)
+        y = torch.zeros((S, M), dtype=torch.float32, device="cuda")
+        side = torch.cuda.Stream()
+        side.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(side):
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=side):
+                for _ in range(3):
+                    batq.batq_linear_w4a4(tr, w, x, y, ws)
+            for _ in range(3):
+                g.replay()
+        torch.cuda.synchronize()
+        codes = torch.empty((S, N // 2), dtype=torch.uint8, device="cuda")
+        sf = torch.empty(batq.batq_sf_bytes(S, N, 1), dtype=torch.uint8, device="cuda")
+        batq.batq_debug_force_quantizer(3)     # the same codes by the other ALU kernel
+        batq.batq_quantize_act(tr, x, codes, sf, 1)
+        y2 = torch.zeros((S, M), dtype=torch.float32, device="cuda")
+        if small:
+            batq.batq_gemm_mxfp4_small_s(codes, sf, w, S, y2, batq.aligned_workspace(batq.batq_gemm_small_s_scratch_bytes(w, S)))
+        else:
+            batq.batq_gemm_mxfp4(codes, sf, w, S, y2)
+    finally:
+        batq.batq_debug_force_quantizer(0)
+        batq.batq_debug_force_small_s_splits(0)
+    assert batq.batq_last_device_status() == 0
+    assert torch.isfinite(y).all() and torch.equal(y, y2)
+
+
 def test_linear_kernel_launches_reports_the_dispatch(batq):
     """1 = the fused kernel (a token or so on a layer whose K slices are short), 2 = quantiser + GEMM."""
     t = synth.make_transform(4096, 3, "baseline")
@@ -959,9 +1005,9 @@ def test_linear_kernel_launches_reports_the_dispatch(batq):
                                             (4096, 4096, 2, 2), (4608, 3584, 1, 2), (1024, 4096, 2, 1), (2304, 4096, 2, 1),
                                             (2432, 4096, 2, 2), (1024, 4096, 3, 2), (1024, 5120, 2, 2)])
 def test_fused_decode_dispatch(batq, M, N, S, launches):
-    """One K-step per CTA: up to four tokens; two: two tokens while no SM has two CTAs (18 x 8 of 148); more: one
-    token; never where the clusters of K splits would
-    fill more than 90 % of the CTA slots (4608 features: 36 x 8 of 296).  The result is the oracle's either way."""
+    """One K-step per CTA: up to four tokens; two: two tokens while no SM has two CTAs (18 x 8 of 148); more:
+    one token; never where the clusters of K splits would fill more than 90 % of the CTA slots (4608
+    features: 36 x 8 of 296).  The result is the oracle's either way."""
     t = synth.make_transform(N, 3, "baseline")
     tr = _mk_transform(batq, t)
     xb, wb = synth.make_activations(S, N, 4), synth.make_weight(M, N, 3)

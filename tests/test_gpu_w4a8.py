@@ -85,6 +85,19 @@ def test_w4a8_few_tokens_gemm_vs_oracle_same_codes(batq, S, M, N, splits):
     assert np.max(np.abs(got - Y) / (Sabs + 1e-30)) < 1e-5
 
 
+@pytest.mark.parametrize("splits", [0, 2])
+@pytest.mark.parametrize("S", [3, 17, 40, 80])
+def test_w4a8_few_tokens_gemm_bf16_output_is_rounded_fp32(batq, S, splits):
+    """Every token tile, features that are no multiple of the four of a 16-byte load."""
+    batq.batq_debug_force_small_s_splits(splits)
+    try:
+        a, _, _ = _gemm_case(batq, S, 261, 1152, 43)
+        b, _, _ = _gemm_case(batq, S, 261, 1152, 43, out_dtype=torch.bfloat16)
+    finally:
+        batq.batq_debug_force_small_s_splits(0)
+    assert np.array_equal(b.astype(np.float32), torch.from_numpy(a.astype(np.float32)).bfloat16().float().numpy())
+
+
 @pytest.mark.parametrize("S,M,N", [(48, 264, 1024), (62, 264, 2048), (64, 264, 2048), (65, 264, 4096), (126, 264, 4096),
                                    (128, 264, 4096), (128, 5008, 8192)])
 def test_w4a8_gemm_on_either_side_of_the_dispatch(batq, S, M, N):
@@ -119,6 +132,82 @@ def test_mxfp8_per_block_quantiser_vs_tensor_cores(batq, S, N, gr, gc, layout):
     assert np.array_equal(out[0][1], out[1][1])
     differ = out[0][0] != out[1][0]
     assert differ.mean() <= 1e-3 and np.abs(out[0][0] - out[1][0]).max() <= 1
+
+
+@pytest.mark.parametrize("layout", [0, 1], ids=["rowmajor", "mma"])
+@pytest.mark.parametrize("mode", [2, 3, 4], ids=["tensorcore", "perblock", "peritem"])
+def test_every_mxfp8_quantiser_on_special_values(batq, mode, layout):
+    """Zero blocks, signed zeros, ties to even at normal and subnormal codes, saturation, 2^+-100 and a subnormal
+    block (identity factors, no clip: the plain MXFP8 of X; a zero's sign bit alone is free)."""
+    N = 256
+    X = np.zeros((6, N), np.float32)
+    blk = np.array([256, 1.0625, -1.0625, 1.1875, 1.9375, 17, 19, -21, 3.875, 2.0 ** -9, 2.0 ** -10, 3 * 2.0 ** -10,
+                    -5 * 2.0 ** -10, 2.0 ** -11, 2.0 ** -6, 17 * 2.0 ** -10, 448, 240, 232, -248, 0.0, -0.0, 30, 34] + [1.5] * 8,
+                   np.float32)
+    X[0, 32:64] = blk
+    X[0, 64:96] = np.array([480, -480, 464, -464, 456, 448, 432, 416] * 4, np.float32)      # saturation on both signs
+    X[1, :32] = -0.0
+    X[1, 64:96] = blk * 2.0 ** -110
+    X[2, :] = np.random.default_rng(0).standard_normal(N).astype(np.float32) * 2.0 ** 100
+    X[3, 96:128] = 2.0 ** -133   # below the normal range of bf16: the scale clamps at 2^-127
+    X[4, 128:160] = -blk * 2.0 ** 20
+    X[5, 0:32] = blk[::-1]
+    xb = synth.f32_to_bf16_bits(X)
+    V = O.bf16_bits_to_f64(xb)
+    assert np.array_equal(V[0], X[0].astype(np.float64))       # the inputs are bf16 values
+    tr = _mk(batq, _identity(N))
+    codes = torch.full((6, N), 0xEE, dtype=torch.uint8, device="cuda")
+    sf = torch.full((batq.batq_sf_bytes(6, N, layout),), 0xEE, dtype=torch.uint8, device="cuda")
+    batq.batq_debug_force_quantizer(mode)
+    try:
+        batq.batq_quantize_act_mxfp8(tr, batq.bits_to_cuda_bf16(xb), codes, sf, layout)
+    finally:
+        batq.batq_debug_force_quantizer(0)
+    h = sf.cpu().numpy()
+    gs = sf_mma_to_rowmajor(h, 6, N // 32) if layout else h.reshape(6, N // 32)
+    gc = codes.cpu().numpy()
+    oc, os_ = O.mxfp8_quantize(V)
+    assert np.array_equal(gs, os_)
+    assert np.array_equal(gc & 0x7F, oc & 0x7F)
+    nz = (oc & 0x7F) != 0
+    assert np.array_equal(gc[nz], oc[nz])
+
+
+@pytest.mark.parametrize("S,M,N", [(5, 264, 1024), (75, 264, 4096), (75, 1024, 14336), (100, 12288, 4096)])
+def test_w4a8_layer_of_few_tokens_equals_its_kernels(batq, S, M, N):
+    """The layer's own choice up to 128 tokens (per-block and thread-per-item ALU quantisers in front of the
+    swapped-operand GEMM and of one CTA per tile), replayed in a graph on a workspace that held garbage: bit for
+    bit the ALU quantiser's codes through the GEMM entry point."""
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(S)
+    tr = _mk(batq, synth.make_transform(N, 3, "baseline"))
+    w = batq.batq_weight_import(torch.randint(0, 256, (M, N // 2), generator=gen, dtype=torch.uint8, device="cuda"),
+                                torch.randint(118, 128, (M, N // 32), generator=gen, dtype=torch.uint8, device="cuda"))
+    x = torch.randn((S, N), generator=gen, device="cuda").bfloat16()
+    ws = batq.aligned_workspace(batq.batq_linear_w4a8_workspace_bytes(w, S))
+    ws.fill_(0xA5)
+    y = torch.zeros((S, M), dtype=torch.bfloat16, device="cuda")
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(side):
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=side):
+            for _ in range(3):
+                batq.batq_linear_w4a8(tr, w, x, y, ws)
+        for _ in range(3):
+            g.replay()
+    torch.cuda.synchronize()
+    codes = torch.empty((S, N), dtype=torch.uint8, device="cuda")
+    sf = torch.empty(batq.batq_sf_bytes(S, N, 1), dtype=torch.uint8, device="cuda")
+    batq.batq_debug_force_quantizer(3)
+    try:
+        batq.batq_quantize_act_mxfp8(tr, x, codes, sf, 1)
+    finally:
+        batq.batq_debug_force_quantizer(0)
+    y2 = torch.zeros((S, M), dtype=torch.bfloat16, device="cuda")
+    batq.batq_gemm_mxfp8_mxfp4(codes, sf, w, S, y2)
+    assert batq.batq_last_device_status() == 0
+    assert torch.isfinite(y.float()).all() and torch.equal(y, y2)
 
 
 @pytest.mark.parametrize("gr,gc,S", [(16, 2, 8), (16, 2, 32), (1, 32, 32), (4, 8, 129)])
