@@ -1124,9 +1124,9 @@ int pick_splits(int64_t m, int64_t n, int64_t s, int sm_count, bool a8 = false) 
 // for any number of tokens.  With up to one row tile of weights an SM, the K-steps of 256 that the splits
 // save an SM count: one for every 5 tokens pays, one for every 9 with MXFP8, whose steps take twice as long.
 // Two CTAs on an SM take as long as their steps one after another, with MXFP8 three quarters of that.
-// Whole layers cold, swapped operands / one CTA per tile: 14336 -> 4096 (saving 40 to 49) 15.0 / 22 us at 75
-// tokens, 17.9 / 22.6 at 128; 4096 -> 12288 (none) 13.9 / 12.1 and 16.3 / 12.2; MXFP8 4096 -> 6144 (10) 11.5 / 12.2
-// at 80 and 13.9 / 12.8 at 128, 14336 -> 10752 (14) 29.3 / 35.7 at 64, 4096 -> 16384 (4) 17.6 / 15.3 at 80.
+// Whole layers cold, swapped operands / one CTA per tile: 14336 -> 4096 (saving 40) 14.6 / 21.5 us at 75
+// tokens, 18.3 / 23.1 at 128; 4096 -> 12288 (none) 13.1 / 11.4 and 15.5 / 11.8; MXFP8 4096 -> 6144 (10) 12.7 / 13.6
+// at 80 and 14.9 / 13.8 at 128, 14336 -> 10240 (14) 29.2 / 35.8 at 64, 4096 -> 16384 (4) 17.8 / 15.5 at 80.
 // With more row tiles than SMs neither splits, and the two lie within 5 % of one another from 75 tokens
 // on; behind a short GEMM the ring of the swapped-operand kernel is full before the activations are there,
 // which is worth 1 us up to 80 tokens (a layer of 4096 / 14336 channels: 54.5 / 55.4 us at 72, 60.8 / 60.1 at 128).
