@@ -335,9 +335,10 @@ batq_status launch_quantize_tc(const batq_transform* t, const void* x, int64_t s
   p.s = s;
   p.n = static_cast<int32_t>(n);
   p.k = static_cast<int32_t>(n / 32);
-  p.n_strips = (p.k + kQtGroups - 1) / kQtGroups;
-  p.n_row_tiles = (s + kQtRows - 1) / kQtRows;
-  p.n_units = p.n_strips * p.n_row_tiles;
+  const int32_t n_strips = (p.k + kQtGroups - 1) / kQtGroups;
+  p.n_row_tiles = static_cast<int32_t>((s + kQtRows - 1) / kQtRows);
+  const int grid = static_cast<int>(std::min<int64_t>(sm_count, static_cast<int64_t>(n_strips) * p.n_row_tiles));
+  p.plan = qt_plan(n_strips, p.n_row_tiles, grid);
   p.pimg = t->d_pimg;
   p.clip_lo = t->d_clip_lo;
   p.clip_hi = t->d_clip_hi;
@@ -355,11 +356,10 @@ batq_status launch_quantize_tc(const batq_transform* t, const void* x, int64_t s
              : make_tmap_2d(&tmap_codes, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, codes, n / 2, s, n / 2, 64, kQtRows,
                             CU_TENSOR_MAP_SWIZZLE_64B);
   if (st != BATQ_OK) return st;
-  if (debug_out == nullptr && layout == BATQ_SF_MMA && p.sf_katoms > p.n_strips) {
+  if (debug_out == nullptr && layout == BATQ_SF_MMA && p.sf_katoms > n_strips) {
     // an odd number of 4-block atoms: keep the padding atom finite
     if (cudaMemsetAsync(scales, 0, batq_sf_bytes(s, n, BATQ_SF_MMA), stream) != cudaSuccess) { cudaGetLastError(); return BATQ_ERR_CUDA; }
   }
-  const int grid = static_cast<int>(std::min<int64_t>(sm_count, p.n_units));
   const bool cl = t->has_clip, dbg = debug_out != nullptr;
   // Launched as a programmatic dependent: if the kernel before it on the stream releases its
   // dependents early (the GEMMs of this library do), the quantiser's CTAs take over the SMs that

@@ -44,13 +44,101 @@ constexpr int kQtStagingBytes = kQtOutBufs * (kQtCodeTileBytes8 + 512);  // code
 constexpr int kQtSmemBytes = kQtStages * kQtStageBytes + 2 * kQtStripImageBytes + kQtStagingBytes + 1024;
 constexpr int kQtTmemCols = kQtDBufs * kQtGroups * 32;  // 4 buffers x 4 blocks x 32 columns = all 512
 
+
+// Which units (128-token row tile, strip of 4 blocks) a CTA works through, and in what order.
+//
+// A CTA keeps to one strip where it can (its block-matrix image stays in shared memory), so what DRAM sees
+// is decided by what the CTAs read at the same time: 256 bytes of each of 128 rows per unit.  With one
+// contiguous range of units per CTA the CTAs were at unrelated rows, and the loads alone ran at 5.0 TB/s
+// (a linear copy kernel: 6.5).  So CTAs go down the rows in step: `per` groups of CTAs for every `group`
+// neighbouring strips, group number q on row tiles q, q + per, ...: whole rows of X at any time.  The CTAs
+// left over (148 of them do not divide by the strips) share the last rows, in ranges.
+// 32768 x 8192 135 -> 111 us, 32768 x 4096 67.5 -> 60, with MXFP8 codes 71.8 -> 65.3; 8192 x 18944 (more strips
+// than CTAs: ranges over groups of strips) 76 -> 69 with groups of 4, 72 without.
+struct QtPlan {                  // of a launch
+  int32_t group;                 // neighbouring strips that go together
+  int32_t strip_groups, n_groups;
+  int32_t per, split;            // walkers per strip group on rows [0, split); per = 0: ranges over everything
+  int32_t units, extra;          // of the ranges: each has `units`, the first `extra` one more
+};
+struct QtWalk {                  // of a CTA
+  int n;                         // units
+  int u0, us;                    // of numbers u0, u0 + us, ...
+  int strip0, group;             // unit u: strip strip0 + (u / height) * group,
+  int row0, height;              //         row tile row0 + u % height
+};
+inline QtPlan qt_plan(int n_strips, int n_row_tiles, int grid) {
+  QtPlan p{};
+  p.group = (n_strips % 4 == 0 && grid % 4 == 0) ? 4 : (n_strips % 2 == 0 && grid % 2 == 0) ? 2 : 1;
+  p.n_groups = grid / p.group;
+  p.strip_groups = n_strips / p.group;
+  p.per = p.n_groups / p.strip_groups;
+  const int rest = p.n_groups - p.per * p.strip_groups;
+  const int64_t units = static_cast<int64_t>(p.strip_groups) * n_row_tiles;   // of a group of CTAs
+  // Rows [0, split) are walked in step, the rest is what the CTAs left over can do meanwhile.
+  p.split = n_row_tiles;
+  int64_t longest = p.per != 0 ? (n_row_tiles + p.per - 1) / p.per : 0;
+  if (p.per != 0 && rest != 0) {
+    longest = INT64_MAX;
+    const int64_t steps = units / p.n_groups;
+    for (int64_t c = steps; c <= steps + 1; ++c) {
+      const int64_t r = c * p.per < n_row_tiles ? c * p.per : n_row_tiles;
+      const int64_t others = (p.strip_groups * (n_row_tiles - r) + rest - 1) / rest, l = (r + p.per - 1) / p.per;
+      if ((others > l ? others : l) < longest) { longest = others > l ? others : l; p.split = static_cast<int32_t>(r); }
+    }
+  }
+  // Ranges: fewer groups of CTAs than of strips, or an uneven split (the last wave counts for more there).
+  const int64_t even = (units + p.n_groups - 1) / p.n_groups;
+  const bool ranges = p.per == 0 || longest * 50 > even * 51;
+  if (ranges) { p.per = 0; p.split = 0; }
+  const int64_t left = static_cast<int64_t>(p.strip_groups) * (n_row_tiles - p.split);
+  const int owners = ranges ? p.n_groups : rest > 0 ? rest : 1;
+  p.units = static_cast<int32_t>(left / owners);
+  p.extra = static_cast<int32_t>(left % owners);
+  return p;
+}
+__host__ __device__ inline QtWalk qt_walk(const QtPlan& p, int n_row_tiles, int cta) {
+  const int at = cta / p.group, in = cta - at * p.group, walkers = p.per * p.strip_groups;
+  QtWalk w;
+  w.group = p.group;
+  if (at < walkers) {
+    w.u0 = at / p.strip_groups;
+    w.us = p.per;
+    w.n = p.split > w.u0 ? (p.split - w.u0 + p.per - 1) / p.per : 0;
+    w.strip0 = (at - w.u0 * p.strip_groups) * p.group + in;
+    w.row0 = 0;
+    w.height = n_row_tiles;
+    return w;
+  }
+  const int q = at - walkers;
+  w.u0 = q * p.units + (q < p.extra ? q : p.extra);
+  w.n = p.units + (q < p.extra ? 1 : 0);
+  w.us = 1;
+  w.strip0 = in;
+  w.row0 = p.split;
+  w.height = n_row_tiles > p.split ? n_row_tiles - p.split : 1;
+  return w;
+}
+// The walk's position, moved on without a division (every role of the CTA keeps one).
+struct QtUnit {
+  int strip, row;
+  __device__ __forceinline__ QtUnit(const QtWalk& w, int skip) : strip(w.strip0), row(w.u0) {
+    if (row >= w.height) { const int s = row / w.height; strip += s * w.group; row -= s * w.height; }
+    advance(w, skip);
+  }
+  __device__ __forceinline__ void advance(const QtWalk& w, int units) {
+    row += units * w.us;
+    while (row >= w.height) { row -= w.height; strip += w.group; }
+  }
+  __device__ __forceinline__ int row_tile(const QtWalk& w) const { return w.row0 + row; }
+};
+
 struct QuantTcParams {
   int64_t s;
   int32_t n;
   int32_t k;             // n / 32
-  int32_t n_strips;      // ceil(k / 4)
-  int64_t n_row_tiles;   // ceil(s / 128)
-  int64_t n_units;       // n_strips * n_row_tiles
+  QtPlan plan;
+  int32_t n_row_tiles;   // ceil(s / 128)
   const uint8_t* pimg;   // [k][3 terms][2048]: P_j^T as bf16 in the MMA's no-swizzle K-major layout
   const float* clip_lo;  // [k] or NULL
   const float* clip_hi;
@@ -179,33 +267,28 @@ quantize_act_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_
   tc_fence_after_sync();
   const uint32_t tmem_base = tmem_base_slot;
 
-  // Units of this CTA: u0, u0 + us, ... below u1; unit u = strip * n_row_tiles + row_tile.  A contiguous
-  // range, so that a CTA keeps its block-matrix image; where there is one strip only there is one image
-  // anyway, and every gridDim.x-th unit is the quicker order (32768 x 128: 5.7 -> 5.2 us).  With several
-  // strips, strips fastest over the CTAs measured 0.5 us better on operands in L2 (2048 x 4096: 8.2 ->
-  // 7.7) but 1 % worse on a layer and 2-7 % worse at 32768 x 8192 on operands from HBM.
-  const int64_t us = p.n_strips == 1 ? gridDim.x : 1;
-  const int64_t u0 = p.n_strips == 1 ? blockIdx.x : p.n_units * blockIdx.x / gridDim.x;
-  const int64_t u1 = p.n_strips == 1 ? p.n_units : p.n_units * (blockIdx.x + 1) / gridDim.x;
+  const QtWalk walk = qt_walk(p.plan, p.n_row_tiles, static_cast<int>(blockIdx.x));
+  const int n_own = walk.n;   // units of this CTA
 
   if (warp == 0) {
     // ---------------------------------------------------------------- TMA producer
     int stage = 0;
     uint32_t phase = 0;
-    int64_t cur_strip = -1;
+    int cur_strip = -1;
     int n_img = 0;  // block-matrix images loaded so far
     bool ok = true;
     int issued = 0;
     bool waited = false;
-    for (int64_t u = u0; u < u1 && ok; u += us) {
-      const int64_t strip = u / p.n_row_tiles;
-      const int row0 = static_cast<int>(u - strip * p.n_row_tiles) * kQtRows;
+    QtUnit at(walk, 0);
+    for (int i = 0; i < n_own && ok; ++i, at.advance(walk, 1)) {
+      const int strip = at.strip;
+      const int row0 = at.row_tile(walk) * kQtRows;
       if (strip != cur_strip) {
         cur_strip = strip;
         const int pb = n_img & 1;
         ok = __all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&p_empty[pb]), ((n_img >> 1) & 1) ^ 1u, &abort_flag));
         if (!ok) break;
-        const int j0 = static_cast<int>(strip) * kQtGroups;
+        const int j0 = strip * kQtGroups;
         const int ng = min(kQtGroups, p.k - j0);
         if (elect_one()) {
           mbar_arrive_expect_tx(smem_u32(&p_full[pb]), static_cast<uint32_t>(ng) * kQtImageBytes);
@@ -226,7 +309,7 @@ quantize_act_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_
       if (elect_one()) {
         const uint32_t bar = smem_u32(&x_full[stage]);
         const uint32_t dst = smem_u32(x_smem + stage * kQtStageBytes);
-        const int col0 = static_cast<int>(strip) * (kQtGroups * 32);
+        const int col0 = strip * (kQtGroups * 32);
         mbar_arrive_expect_tx(bar, kQtStageBytes);
         tma_load_2d(dst, &tmap_x, col0, row0, bar);
         tma_load_2d(dst + kQtBoxBytes, &tmap_x, col0 + 64, row0, bar);
@@ -249,12 +332,12 @@ quantize_act_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_
     const uint64_t b_desc0 = make_smem_desc(smem_u32(img_smem), 128, 512, 0); // no swizzle: LBO 128 (K), SBO 512 (N)
     int stage = 0;
     uint32_t phase = 0;
-    int64_t cur_strip = -1;
+    int cur_strip = -1;
     int n_img = 0;
-    int it = 0;
     bool ok = true;
-    for (int64_t u = u0; u < u1 && ok; u += us, ++it) {
-      const int64_t strip = u / p.n_row_tiles;
+    QtUnit at(walk, 0);
+    for (int it = 0; it < n_own && ok; ++it, at.advance(walk, 1)) {
+      const int strip = at.strip;
       if (strip != cur_strip) {
         if (cur_strip >= 0 && elect_one()) tc_commit(smem_u32(&p_empty[(n_img - 1) & 1]));  // old image no longer read
         cur_strip = strip;
@@ -269,7 +352,7 @@ quantize_act_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_
       ok = __all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&x_full[stage]), phase, &abort_flag));
       if (!ok) break;
       tc_fence_after_sync();
-      const int ng = min(kQtGroups, p.k - static_cast<int>(strip) * kQtGroups);
+      const int ng = min(kQtGroups, p.k - strip * kQtGroups);
       const uint64_t a_stage = a_desc0 + static_cast<uint32_t>((stage * kQtStageBytes) >> 4);
       const uint64_t b_img = b_desc0 + static_cast<uint32_t>((pb * kQtStripImageBytes) >> 4);
       const uint32_t d0 = tmem_base + buf * (kQtGroups * 32);
@@ -297,13 +380,13 @@ quantize_act_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_
   } else if (warp == 2 + kQtQuantWarps) {
     // ---------------------------------------------------------------- store warp
     if (!DEBUG_OUT && lane == 0) {
-      int it = 0;
-      for (int64_t u = u0; u < u1; u += us, ++it) {
-        const int64_t strip = u / p.n_row_tiles;
-        const int64_t row_tile = u - strip * p.n_row_tiles;
+      QtUnit at(walk, 0);
+      for (int it = 0; it < n_own; ++it, at.advance(walk, 1)) {
+        const int strip = at.strip;
+        const int64_t row_tile = at.row_tile(walk);
         const int sb = it % kQtOutBufs;
         if (!mbar_wait(smem_u32(&t_full[sb]), static_cast<uint32_t>(it / kQtOutBufs) & 1u, &abort_flag)) break;
-        tma_store_2d(&tmap_codes, static_cast<int>(strip) * (kQtGroups * (FP8 ? 32 : 16)),
+        tma_store_2d(&tmap_codes, strip * (kQtGroups * (FP8 ? 32 : 16)),
                      static_cast<int>(row_tile) * kQtRows, smem_u32(staging + sb * kQtCodeTileBytes8));
         if (p.sf_layout != 0)
           bulk_s2g(p.scales + (row_tile * p.sf_katoms + strip) * 512,
@@ -322,10 +405,10 @@ quantize_act_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_
     const int quad = warp & 3;          // tensor-memory lanes [32 quad, 32 quad + 32)
     const int grp = qw >> 3;            // takes the units of this CTA with it % 2 == grp
     const int half = (qw & 7) >> 2;     // blocks 2 half and 2 half + 1 of the unit
-    for (int it = grp; u0 + it * us < u1; it += 2) {
-      const int64_t u = u0 + it * us;
-      const int64_t strip = u / p.n_row_tiles;
-      const int64_t row_tile = u - strip * p.n_row_tiles;
+    QtUnit at(walk, grp);
+    for (int it = grp; it < n_own; it += 2, at.advance(walk, 2)) {
+      const int strip = at.strip;
+      const int64_t row_tile = at.row_tile(walk);
       const int buf = it & (kQtDBufs - 1);
       bool ok = mbar_wait(smem_u32(&d_full[buf]), (it >> 2) & 1u, &abort_flag);
       ok = __all_sync(0xFFFFFFFFu, ok);
@@ -343,7 +426,7 @@ quantize_act_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_
 #pragma unroll 1
      for (int e = 0; e < 2; ++e) {
       const int g = 2 * half + e;
-      const int j = static_cast<int>(strip) * kQtGroups + g;
+      const int j = strip * kQtGroups + g;
       const uint32_t taddr = tmem_base + buf * (kQtGroups * 32) + g * 32 + (static_cast<uint32_t>(quad * 32) << 16);
       uint32_t v[32];
       tmem_ld_32x32b_x32(taddr, v);
