@@ -39,10 +39,11 @@ int32_t batq_debug_pair_schedule(int64_t s, int64_t m, int64_t n, int32_t sm_cou
 int32_t batq_debug_wide_schedule(int64_t s, int64_t m, int64_t n, int32_t sm_count, int32_t pair,
                                  int32_t* tiles, int32_t max_tiles);
 
-/* Which prefill GEMM kernel later calls use.  0 = automatic (CTA pairs sharing a 256-token tile
- * for s > 128 -- with tiles of up to 256 features and two accumulators, or tiles of up to 448
- * features and one, whichever the cost model expects to finish first --, one CTA per 128-token
- * tile otherwise; batq_gemm_mxfp8_mxfp4 takes the swapped-operand kernel up to 48 tokens, and up to 128
+/* Which prefill GEMM kernel later calls use.  0 = automatic (up to 128 tokens, and where the device
+ * has an SM for every tile at once or an odd number of row tiles fills its waves, one CTA per
+ * 128-token tile; else CTA pairs sharing a 256-token tile, with tiles of up to 256 features and two
+ * accumulators, or tiles of up to 448 features and one, whichever the cost model expects to finish
+ * first; batq_gemm_mxfp8_mxfp4 takes the swapped-operand kernel up to 48 tokens, and up to 128
  * where its K splits pay), 1 = always one CTA per tile, 2 = always CTA pairs with two accumulators,
  * 3 = always CTA pairs with wide tiles (batq_debug_force_tile_width then takes any multiple of 64
  * up to 448 and makes every column that wide). */

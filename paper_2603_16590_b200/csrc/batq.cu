@@ -631,6 +631,28 @@ int pick_bn(int64_t s, int64_t m, int64_t n, int sm_count) {
   return c256 <= c128 ? 256 : 128;
 }
 
+// Above 128 tokens: the tile width with which the kernels of one CTA per 128-token tile take the layer, or 0 for
+// the CTA pairs.  A pair shares a weight tile between 256 rows, which is what counts once the tiles go into
+// several waves; in a single wave what counts is how many SMs there is a tile for, how many of its rows are
+// padding (333 tokens: 384 rows in tiles of 128, 512 in pairs), and 1 us less for the cluster launch.  Whole
+// layers back to back, pairs / one CTA per tile:
+//   one wave of 128-wide tiles: 4096 -> 6144 14.4 / 12.5 us at 333 tokens (MXFP8 18.7 / 16.4), 4096 -> 4096 13.9 / 12.4 at
+//     512 (18.1 / 16.4), 14336 -> 4096 26.5 / 24.2 at 333 (40.2 / 37.4), 2048 -> 2048 11.7 / 10.4 at 1024 (13.9 / 12.6), 18944 -> 3584
+//     35.0 / 31.8 at 640 (54.9 / 50.0); 64-wide tiles on short K (2048 -> 2048 at 200 9.4 / 8.5, 128-wide 8.9; 14336 -> 4096 23.8,
+//     128-wide 22.9);
+//   one wave of 192-wide tiles, K of 4096: 4096 -> 6144 14.8 / 13.9 at 512, 4096 -> 4096 15.2 / 14.5 at 768, but 14336 ->
+//     4096 29.3 / 30.7 at 640: pairs move fewer bytes per K-step;
+//   an odd number of row tiles and full waves of 256-wide ones: 3584 -> 37888 35.1 / 31.9 at 333 (53.6 / 47.2), 640
+//     tokens 47.7 / 47.5 (78.0 / 75.1); waves less than full: 4096 -> 28672 29.7 / 32.1 at 257.
+int one_cta_width(int64_t s, int64_t m, int64_t n, int sm_count, bool a8) {
+  const int64_t mt = (s + kBM - 1) / kBM, k_steps = (n + 255) / 256;
+  auto tiles = [&](int bn) { return mt * ((m + bn - 1) / bn); };
+  if (tiles(128) <= sm_count) return (!a8 && tiles(128) * 2 <= sm_count && m > 64 && k_steps <= 12) ? 64 : 128;
+  if (!a8 && tiles(192) <= sm_count && k_steps <= 24) return 192;
+  const int64_t waves = (tiles(256) + sm_count - 1) / sm_count;
+  return (mt & 1) != 0 && tiles(256) * 100 >= waves * sm_count * 97 ? 256 : 0;
+}
+
 std::atomic<int> g_force_gemm_kernel{0};  // tuning hook: 0 = automatic, 1 = one CTA per tile, 2 = CTA pairs (two accumulators), 3 = CTA pairs (wide tiles)
 
 // The schedule of the CTA-pair kernel for an s x m output with k_steps K-steps: the segments of
@@ -1023,9 +1045,12 @@ batq_status launch_gemm(const void* x_codes, const void* x_sf, const batq_weight
   if (st != BATQ_OK) return st;
   // CTA pairs need at least two 128-token tiles to pay, and wide enough a layer for their tiles.
   const int force_gemm = g_force_gemm_kernel.load(std::memory_order_relaxed);
-  const bool use_pair = force_gemm == 2 || force_gemm == 3 || (force_gemm == 0 && s > 128 && w->m >= 192);
+  const bool free_choice = force_gemm == 0 && s > 128 && w->m >= 192;
+  const int cta_bn = free_choice && g_force_bn.load(std::memory_order_relaxed) == 0
+                         ? one_cta_width(s, w->m, w->n, info->sm_count, false) : 0;
+  const bool use_pair = force_gemm == 2 || force_gemm == 3 || (free_choice && cta_bn == 0);
   if (use_pair) return launch_gemm_pair(x_codes, x_sf, w, s, y, bf, ldy, stream, info->sm_count, tmap_a, tmap_y, m16, dependent);
-  const int bn = pick_bn(s, w->m, w->n, info->sm_count);
+  const int bn = cta_bn != 0 ? cta_bn : pick_bn(s, w->m, w->n, info->sm_count);
   GemmParams p{};
   p.sfa = static_cast<const uint8_t*>(x_sf);
   p.sfb = w->scales;
@@ -1456,7 +1481,10 @@ batq_status launch_gemm_w4a8(const void* x_codes8, const void* x_sf, const batq_
   // the rule here; the two-accumulator kernel keeps the layers where a pair has at most two tiles
   // whichever way the features are cut.
   const int force_gemm = g_force_gemm_kernel.load(std::memory_order_relaxed);
-  if (force_gemm == 2 || force_gemm == 3 || (force_gemm == 0 && s > 128 && w->m >= 192)) {
+  const bool free_choice = force_gemm == 0 && s > 128 && w->m >= 192;
+  const int cta_bn = free_choice && g_force_bn.load(std::memory_order_relaxed) == 0
+                         ? one_cta_width(s, w->m, w->n, info->sm_count, true) : 0;
+  if (force_gemm == 2 || force_gemm == 3 || (free_choice && cta_bn == 0)) {
     CUtensorMap tmap_sfa, tmap_y64;
     std::memset(&tmap_y64, 0, sizeof(tmap_y64));
     st = make_sf_tmap(&tmap_sfa, x_sf, (s + 127) / 128, w->katoms, 1);
@@ -1533,6 +1561,7 @@ batq_status launch_gemm_w4a8(const void* x_codes8, const void* x_sf, const batq_
   const int force_bn = g_force_bn.load(std::memory_order_relaxed);
   int bn = (w->m <= 128 || waves(128) * 128 * 1.2 < waves(256) * 256) ? 128 : 256;
   if (force_bn == 128 || force_bn == 256) bn = force_bn;
+  else if (cta_bn != 0) bn = cta_bn;
   W4A8Params p{};
   p.sfa = static_cast<const uint8_t*>(x_sf);
   p.sfb = w->scales;
