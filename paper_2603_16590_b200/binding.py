@@ -8,6 +8,8 @@ fails loudly when the shared library is missing.
 from __future__ import annotations
 
 import ctypes as C
+import importlib.machinery
+import importlib.util
 import os
 
 import numpy as np
@@ -20,6 +22,8 @@ STATUS_NAMES = {0: "OK", 1: "ERR_NULL", 2: "ERR_SHAPE", 3: "ERR_ALIGN", 4: "ERR_
                 5: "ERR_WORKSPACE", 6: "ERR_SINGULAR", 7: "ERR_CUDA", 8: "ERR_TIMEOUT"}
 
 _LIB = None
+_CALL = None     # csrc/pycall.c: the calls a program makes per layer, without ctypes' conversions
+_ADDRESS = {}    # entry point -> address, for _CALL
 _P, _I64, _I32, _SZ = C.c_void_p, C.c_int64, C.c_int32, C.c_size_t
 
 # name -> (restype, argtypes); must list every symbol include/batq.h and include/batq_debug.h declare
@@ -99,8 +103,22 @@ def load():
         for name, (res, args) in SIGNATURES.items():
             fn = getattr(lib, name)
             fn.restype, fn.argtypes = res, args
+        _load_call_shim(lib)
         _LIB = lib
     return _LIB
+
+
+def _load_call_shim(lib):
+    global _CALL
+    path = os.path.join(os.path.dirname(os.path.abspath(__file__)), "_pycall.so")
+    if not os.path.exists(path):
+        raise FileNotFoundError(f"{path} not found: run `python -m paper_2603_16590_b200.build`")
+    loader = importlib.machinery.ExtensionFileLoader("_pycall", path)
+    _CALL = importlib.util.module_from_spec(importlib.util.spec_from_loader("_pycall", loader))
+    loader.exec_module(_CALL)
+    _CALL.setup(torch.float32)
+    for name in ("batq_linear_w4a4", "batq_linear_w4a8", "batq_quantize_act", "batq_quantize_act_mxfp8"):
+        _ADDRESS[name] = C.cast(getattr(lib, name), _P).value
 
 
 def _check(status: int, where: str):
@@ -120,6 +138,27 @@ def _stream():
     # the handle of torch.cuda.current_stream() without the Python object around it: 0.3 us instead of 3.4
     # of a decode call's 9.4 to 11.5
     return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+
+
+def _handle(h):   # of a Transform or Weight; NULL for none, or one that has been closed
+    return h.handle.value if h and h.handle else 0
+
+
+def _quantise(name, t, x, codes, scales, scale_layout, ld, s, n):
+    if _LIB is None:
+        load()
+    if ld is None and s is None and n is None:
+        return _CALL.quantise(_ADDRESS[name], _handle(t), x, codes, scales, scale_layout, _stream())
+    s = x.shape[0] if s is None else s
+    n = x.shape[1] if n is None else n
+    ld = x.stride(0) if ld is None else ld
+    return getattr(_LIB, name)(t.handle if t else None, _ptr(x), s, n, ld, _ptr(codes), _ptr(scales), scale_layout, _stream())
+
+
+def _linear(name, t, w, x, y, workspace):
+    if _LIB is None:
+        load()
+    return _CALL.linear(_ADDRESS[name], _handle(t), _handle(w), x, y, workspace, _stream())
 
 
 def _f32(a):
@@ -171,22 +210,12 @@ def batq_weight_bytes(m, n) -> int:
 
 def batq_quantize_act(t, x, codes, scales, scale_layout=SF_ROWMAJOR, ld=None, s=None, n=None):
     """x: bf16 (or int16 bit-pattern) CUDA tensor [s, n]; codes / scales: uint8 CUDA buffers."""
-    s = x.shape[0] if s is None else s
-    n = x.shape[1] if n is None else n
-    ld = x.stride(0) if ld is None else ld
-    st = load().batq_quantize_act(t.handle if t else None, _ptr(x), s, n, ld, _ptr(codes), _ptr(scales),
-                                  scale_layout, _stream())
-    _check(st, "batq_quantize_act")
+    _check(_quantise("batq_quantize_act", t, x, codes, scales, scale_layout, ld, s, n), "batq_quantize_act")
 
 
 def batq_quantize_act_mxfp8(t, x, codes, scales, scale_layout=SF_ROWMAJOR, ld=None, s=None, n=None):
     """As batq_quantize_act with E4M3 codes: codes is a uint8 CUDA buffer of s * n bytes."""
-    s = x.shape[0] if s is None else s
-    n = x.shape[1] if n is None else n
-    ld = x.stride(0) if ld is None else ld
-    st = load().batq_quantize_act_mxfp8(t.handle if t else None, _ptr(x), s, n, ld, _ptr(codes), _ptr(scales),
-                                        scale_layout, _stream())
-    _check(st, "batq_quantize_act_mxfp8")
+    _check(_quantise("batq_quantize_act_mxfp8", t, x, codes, scales, scale_layout, ld, s, n), "batq_quantize_act_mxfp8")
 
 
 def batq_debug_transform_clip_f32(t, x, out):
@@ -269,10 +298,7 @@ def batq_linear_w4a8_workspace_bytes(w: Weight, s) -> int:
 
 
 def batq_linear_w4a8(t, w: Weight, x, y, workspace):
-    dt = F32 if y.dtype == torch.float32 else BF16
-    st = load().batq_linear_w4a8(t.handle if t else None, w.handle, _ptr(x), x.shape[0], x.stride(0), _ptr(y), dt,
-                                 y.stride(0), _ptr(workspace), workspace.numel(), _stream())
-    _check(st, "batq_linear_w4a8")
+    _check(_linear("batq_linear_w4a8", t, w, x, y, workspace), "batq_linear_w4a8")
 
 
 def batq_gemm_small_s_scratch_bytes(w: Weight, s) -> int:
@@ -353,10 +379,7 @@ def aligned_workspace(nbytes, device="cuda"):
 
 
 def batq_linear_w4a4(t, w: Weight, x, y, workspace):
-    dt = F32 if y.dtype == torch.float32 else BF16
-    st = load().batq_linear_w4a4(t.handle if t else None, w.handle, _ptr(x), x.shape[0], x.stride(0), _ptr(y), dt,
-                                 y.stride(0), _ptr(workspace), workspace.numel(), _stream())
-    _check(st, "batq_linear_w4a4")
+    _check(_linear("batq_linear_w4a4", t, w, x, y, workspace), "batq_linear_w4a4")
 
 
 def batq_linear_w4a4_host(t, w: Weight, x_host, y_host, x_stage, y_stage, workspace):

@@ -4,10 +4,13 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 LIB = os.path.join(HERE, "libbatq.so")
+CALL_LIB = os.path.join(HERE, "_pycall.so")   # CPython shim of the binding's calls
+CALL_SOURCE = os.path.join(HERE, "csrc", "pycall.c")
 SOURCES = [os.path.join(HERE, "csrc", "batq.cu")]
 DEPS = [os.path.join(HERE, "csrc", f) for f in os.listdir(os.path.join(HERE, "csrc"))] + [
     os.path.join(ROOT, "include", "batq.h")]
@@ -20,8 +23,19 @@ def nvcc_command(extra=()):
             "-I", os.path.join(HERE, "csrc"), *extra, "-o", LIB, *SOURCES]
 
 
+def _build_call_shim(force: bool):
+    if not force and os.path.exists(CALL_LIB) and os.path.getmtime(CALL_SOURCE) <= os.path.getmtime(CALL_LIB):
+        return
+    res = subprocess.run(["gcc", "-O2", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], "-o", CALL_LIB, CALL_SOURCE],
+                         capture_output=True, text=True)
+    if res.returncode != 0:
+        sys.stderr.write(res.stderr)
+        raise RuntimeError("gcc failed building _pycall.so")
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compiles libbatq.so if it is missing or older than its sources; returns its path."""
+    """Compiles libbatq.so (and the binding's shim) if missing or older than their sources; returns libbatq.so's path."""
+    _build_call_shim(force)
     if not force and os.path.exists(LIB):
         t = os.path.getmtime(LIB)
         if all(os.path.getmtime(d) <= t for d in DEPS):
