@@ -39,6 +39,7 @@
 
 namespace batq {
 
+constexpr int kPfDBufs = 4;                    // accumulator buffers of the quantise phase
 constexpr int kPfThreads = kQtThreads;        // 19 warps: producer, MMA issuer, 16 quantiser warps, store warp
 constexpr int kPfXStages = 3;
 constexpr int kPfOutBufs = 3;
@@ -132,8 +133,8 @@ linear_prefill_fused_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
   __shared__ __align__(8) uint64_t x_empty[kPfXStages];   // both CTAs: the MMAs have read the stage
   __shared__ __align__(8) uint64_t p_full[2];             // leader: both CTAs' halves of a strip's block matrices
   __shared__ __align__(8) uint64_t p_empty[2];            // both CTAs
-  __shared__ __align__(8) uint64_t d_full[kQtDBufs];      // both CTAs: accumulators of a unit complete
-  __shared__ __align__(8) uint64_t d_empty[kQtDBufs];     // leader: read out by the quantiser warps of both CTAs
+  __shared__ __align__(8) uint64_t d_full[kPfDBufs];      // both CTAs: accumulators of a unit complete
+  __shared__ __align__(8) uint64_t d_empty[kPfDBufs];     // leader: read out by the quantiser warps of both CTAs
   __shared__ __align__(8) uint64_t t_full[kPfOutBufs];    // per CTA: staging tile complete
   __shared__ __align__(8) uint64_t t_empty[kPfOutBufs];   // per CTA: staging tile read out by its stores
   __shared__ __align__(8) uint64_t q_drain;               // leader: all phase-1 MMAs done
@@ -166,7 +167,7 @@ linear_prefill_fused_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
   if (tid == 0) {
     for (int i = 0; i < kPfXStages; ++i) { mbar_init(smem_u32(&x_full[i]), 1); mbar_init(smem_u32(&x_empty[i]), 1); }
     for (int i = 0; i < 2; ++i) { mbar_init(smem_u32(&p_full[i]), 1); mbar_init(smem_u32(&p_empty[i]), 1); }
-    for (int i = 0; i < kQtDBufs; ++i) {
+    for (int i = 0; i < kPfDBufs; ++i) {
       mbar_init(smem_u32(&d_full[i]), 1);
       mbar_init(smem_u32(&d_empty[i]), kQtQuantWarps);     // 8 warps of a group in each CTA
     }
@@ -265,7 +266,7 @@ linear_prefill_fused_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
           ++n_img;
         }
         const int pb = (n_img - 1) & 1;
-        const int buf = it & (kQtDBufs - 1);
+        const int buf = it & (kPfDBufs - 1);
         ok = __all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&d_empty[buf]), ((it >> 2) & 1u) ^ 1u, &abort_flag));
         if (!ok) break;
         ok = __all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&x_full[stage]), phase, &abort_flag));
@@ -344,7 +345,7 @@ linear_prefill_fused_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
     for (int it = grp; u0 + it < u1; it += 2) {
       const int u = u0 + it;
       const int strip = u / p.m_pairs;
-      const int buf = it & (kQtDBufs - 1);
+      const int buf = it & (kPfDBufs - 1);
       bool ok = mbar_wait(smem_u32(&d_full[buf]), (it >> 2) & 1u, &abort_flag);
       ok = __all_sync(0xFFFFFFFFu, ok);
       if (!ok) break;

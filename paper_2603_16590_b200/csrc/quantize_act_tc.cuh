@@ -4,9 +4,13 @@
 // x~ = x P_j (Eq. 1) is a dense 32 x 32 contraction per block.  The ALU version of
 // this kernel (quantize_act.cuh, the Kronecker-factored form of Eq. 2) is bound by
 // instruction issue, not by HBM, so here the contraction runs as tcgen05.mma
-// (kind::f16, bf16 x bf16 -> fp32): A = a 128-token x 32-channel tile of X exactly
-// as TMA lands it in shared memory, B = P_j^T split into three bf16 terms
-// (hi + mid + lo reproduce the fp32 entries), D = 128 x 32 fp32 in tensor memory.
+// (kind::f16, bf16 x bf16 -> fp32): A = a 128-token x 32-channel tile of X, B = P_j^T split
+// into three bf16 terms (hi + mid + lo reproduce the fp32 entries), D = 128 x 32 fp32 in tensor memory.
+// A goes from where TMA lands it in shared memory into tensor memory once (tcgen05.cp) and the six MMAs of a
+// block read it there: an MMA this narrow (32 columns, 17 cycles of arithmetic) takes as long as its operands
+// take to be fetched from shared memory, some 85 cycles for 5 KiB, and 24 of them were what a unit waited for
+// (with one term instead of three 32768 x 8192 ran at the time of its DRAM traffic).  32768 x 8192 124.5 -> 117 us,
+// 32768 x 4096 63 -> 58, with MXFP8 codes 70 -> 65.5, 2048 x 14336 16.8 -> 16.1; the same codes bit for bit.
 // The accumulator row of a token is then read by one thread, which clips (Eq. 3-4),
 // derives the shared scale, rounds to E2M1 and stores 16 code bytes + 1 scale byte.
 //
@@ -39,10 +43,13 @@ constexpr int kQtThreads = (3 + kQtQuantWarps) * 32;  // + TMA producer, MMA iss
 constexpr int kQtCodeTileBytes = kQtRows * kQtGroups * 16;  // 4-bit codes of one unit: 128 rows x 64 bytes
 constexpr int kQtCodeTileBytes8 = 2 * kQtCodeTileBytes;     // 8-bit codes: 128 rows x 128 bytes
 constexpr int kQtOutBufs = 4;   // staging buffers between the quantiser warps and the store warp
-constexpr int kQtDBufs = 4;     // accumulator buffers in tensor memory: two per group of quantiser warps
+constexpr int kQtDBufs = 3;     // accumulator buffers in tensor memory
+constexpr int kQtABufs = 2;     // X of a unit in tensor memory
+constexpr int kQtACols = kQtGroups * 16;      // 64 columns of two bf16
 constexpr int kQtStagingBytes = kQtOutBufs * (kQtCodeTileBytes8 + 512);  // code tiles (sized for 8-bit), scale atoms
 constexpr int kQtSmemBytes = kQtStages * kQtStageBytes + 2 * kQtStripImageBytes + kQtStagingBytes + 1024;
-constexpr int kQtTmemCols = kQtDBufs * kQtGroups * 32;  // 4 buffers x 4 blocks x 32 columns = all 512
+constexpr int kQtTmemCols = 512;   // accumulators 3 x 128, X 2 x 64
+static_assert(kQtDBufs * kQtGroups * 32 + kQtABufs * kQtACols <= kQtTmemCols, "tensor memory budget");
 
 
 // Which units (128-token row tile, strip of 4 blocks) a CTA works through, and in what order.
@@ -155,14 +162,19 @@ __host__ __device__ constexpr uint32_t f16_idesc_bf16(int M, int N) {
          (static_cast<uint32_t>(M >> 4) << 24);
 }
 
-__device__ __forceinline__ void tc_mma_f16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                           uint32_t accumulate) {
+// A in tensor memory: lane = row, a column = two consecutive elements of K.
+__device__ __forceinline__ void tc_mma_f16_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
+                                              uint32_t accumulate) {
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
+      "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
       : "memory");
+}
+// shared -> tensor memory: 128 rows x 256 bits (8 columns), the rows laid out as an MMA operand's.
+__device__ __forceinline__ void tc_cp_128x256b(uint32_t taddr, uint64_t sdesc) {
+  asm volatile("tcgen05.cp.cta_group::1.128x256b [%0], %1;" ::"r"(taddr), "l"(sdesc) : "memory");
 }
 
 __device__ __forceinline__ void bulk_s2g(void* dst, uint32_t src_smem, uint32_t bytes) {
@@ -346,8 +358,8 @@ quantize_act_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_
         ++n_img;
       }
       const int pb = (n_img - 1) & 1;
-      const int buf = it & (kQtDBufs - 1);
-      ok = __all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&d_empty[buf]), ((it >> 2) & 1u) ^ 1u, &abort_flag));
+      const int buf = it % kQtDBufs;
+      ok = __all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&d_empty[buf]), (static_cast<uint32_t>(it / kQtDBufs) & 1u) ^ 1u, &abort_flag));
       if (!ok) break;
       ok = __all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&x_full[stage]), phase, &abort_flag));
       if (!ok) break;
@@ -356,22 +368,26 @@ quantize_act_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_
       const uint64_t a_stage = a_desc0 + static_cast<uint32_t>((stage * kQtStageBytes) >> 4);
       const uint64_t b_img = b_desc0 + static_cast<uint32_t>((pb * kQtStripImageBytes) >> 4);
       const uint32_t d0 = tmem_base + buf * (kQtGroups * 32);
+      const uint32_t a_tmem = tmem_base + kQtDBufs * (kQtGroups * 32) + (it & 1) * kQtACols;
       if (elect_one()) {
+        // X into tensor memory first, 16 channels (32 bytes a row) at a time; cp and mma of one thread
+        // execute in issue order.
+#pragma unroll
+        for (int c = 0; c < 2 * kQtGroups; ++c)   // channels 16 c .. 16 c + 15: box c / 4, byte offset (c % 4) * 32 of its rows
+          tc_cp_128x256b(a_tmem + 8 * c, a_stage + static_cast<uint32_t>(((c >> 2) * kQtBoxBytes + (c & 3) * 32) >> 4));
+        tc_commit(smem_u32(&x_empty[stage]));
 #pragma unroll
         for (int g = 0; g < kQtGroups; ++g) {
           if (g < ng) {
-            // block g lives in box g / 2 at byte offset (g % 2) * 64 of each 128-byte row
-            const uint64_t a_g = a_stage + static_cast<uint32_t>(((g >> 1) * kQtBoxBytes + (g & 1) * 64) >> 4);
             const uint64_t b_g = b_img + static_cast<uint32_t>((g * kQtImageBytes) >> 4);
 #pragma unroll
             for (int t = 2; t >= 0; --t)  // smallest term first
 #pragma unroll
               for (int kk = 0; kk < 2; ++kk)
-                tc_mma_f16(d0 + g * 32, a_g + 2 * kk, b_g + static_cast<uint32_t>((t * kQtTermBytes + kk * 256) >> 4),
-                           idesc, (t == 2 && kk == 0) ? 0u : 1u);
+                tc_mma_f16_ta(d0 + g * 32, a_tmem + g * 16 + 8 * kk, b_g + static_cast<uint32_t>((t * kQtTermBytes + kk * 256) >> 4),
+                              idesc, (t == 2 && kk == 0) ? 0u : 1u);
           }
         }
-        tc_commit(smem_u32(&x_empty[stage]));
         tc_commit(smem_u32(&d_full[buf]));
       }
       if (++stage == kQtStages) { stage = 0; phase ^= 1u; }
@@ -409,8 +425,8 @@ quantize_act_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_
     for (int it = grp; it < n_own; it += 2, at.advance(walk, 2)) {
       const int strip = at.strip;
       const int64_t row_tile = at.row_tile(walk);
-      const int buf = it & (kQtDBufs - 1);
-      bool ok = mbar_wait(smem_u32(&d_full[buf]), (it >> 2) & 1u, &abort_flag);
+      const int buf = it % kQtDBufs;
+      bool ok = mbar_wait(smem_u32(&d_full[buf]), static_cast<uint32_t>(it / kQtDBufs) & 1u, &abort_flag);
       ok = __all_sync(0xFFFFFFFFu, ok);
       if (!ok) break;
       tc_fence_after_sync();
