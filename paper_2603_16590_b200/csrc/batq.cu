@@ -633,24 +633,37 @@ int pick_bn(int64_t s, int64_t m, int64_t n, int sm_count) {
 
 // Above 128 tokens: the tile width with which the kernels of one CTA per 128-token tile take the layer, or 0 for
 // the CTA pairs.  A pair shares a weight tile between 256 rows, which is what counts once the tiles go into
-// several waves; in a single wave what counts is how many SMs there is a tile for, how many of its rows are
-// padding (333 tokens: 384 rows in tiles of 128, 512 in pairs), and 1 us less for the cluster launch.  Whole
-// layers back to back, pairs / one CTA per tile:
+// several waves and K is long; else it counts how many SMs there is a tile for, how many of its rows are padding
+// (333 tokens: 384 rows in tiles of 128, 512 in pairs), and 1 us less for the cluster launch.  Whole layers back
+// to back, pairs / one CTA per tile:
 //   one wave of 128-wide tiles: 4096 -> 6144 14.4 / 12.5 us at 333 tokens (MXFP8 18.7 / 16.4), 4096 -> 4096 13.9 / 12.4 at
 //     512 (18.1 / 16.4), 14336 -> 4096 26.5 / 24.2 at 333 (40.2 / 37.4), 2048 -> 2048 11.7 / 10.4 at 1024 (13.9 / 12.6), 18944 -> 3584
 //     35.0 / 31.8 at 640 (54.9 / 50.0); 64-wide tiles on short K (2048 -> 2048 at 200 9.4 / 8.5, 128-wide 8.9; 14336 -> 4096 23.8,
 //     128-wide 22.9);
-//   one wave of 192-wide tiles, K of 4096: 4096 -> 6144 14.8 / 13.9 at 512, 4096 -> 4096 15.2 / 14.5 at 768, but 14336 ->
-//     4096 29.3 / 30.7 at 640: pairs move fewer bytes per K-step;
-//   an odd number of row tiles and full waves of 256-wide ones: 3584 -> 37888 35.1 / 31.9 at 333 (53.6 / 47.2), 640
-//     tokens 47.7 / 47.5 (78.0 / 75.1); waves less than full: 4096 -> 28672 29.7 / 32.1 at 257.
+//   K up to 1024 (a pair's time between tiles is most of a tile there): 512 -> 4096 10.0 / 8.2 at 1024 tokens, 27.2 / 22.4 at
+//     8192, 512 -> 16384 57.7 / 47.0 at 6000, 1024 -> 4096 14.5 / 12.9 at 2048, but 1024 -> 16384 48.9 / 50.3 at 4096 (19 waves) and
+//     2048 -> 4096 17.1 / 17.8 at 2048; 192-wide tiles from four waves on; with MXFP8 the K-steps are twice as many
+//     (1024 -> 4096 16.2 / 16.9 at 2048);
+//   K up to 6144, one wave of 192- or most of one of 256-wide tiles, or two or three nearly full of 192-wide ones on K up
+//     to 3072: 4096 -> 6144 14.8 / 13.9 at 512, 5120 -> 7168 20.4 / 17.7 at 600, 3584 -> 4608 16.0 / 15.4 at 900, 2560 -> 10240 16.4 / 15.4 at 600,
+//     but 14336 -> 4096 29.3 / 30.7 at 640, 5120 -> 7168 17.1 / 17.2 at 450 (112 tiles): pairs move fewer bytes per K-step;
+//   three row tiles and full waves of 256-wide ones: 3584 -> 37888 35.1 / 31.9 at 333 (53.6 / 47.2), 5120 -> 37888 43.6 / 40.0
+//     (71.3 / 62.0); waves less than full: 4096 -> 28672 29.7 / 32.1 at 257; five row tiles: 60.4 / 60.5.
+// On 17 widths x 14 token counts (129 to 3000) 0.958 of the pairs' time with MXFP4, never above it; the best of all
+// widths 0.954.  MXFP8 0.972 and 0.965.
 int one_cta_width(int64_t s, int64_t m, int64_t n, int sm_count, bool a8) {
-  const int64_t mt = (s + kBM - 1) / kBM, k_steps = (n + 255) / 256;
+  const int64_t mt = (s + kBM - 1) / kBM, k_steps = (n + 255) / 256, sms = sm_count;
   auto tiles = [&](int bn) { return mt * ((m + bn - 1) / bn); };
-  if (tiles(128) <= sm_count) return (!a8 && tiles(128) * 2 <= sm_count && m > 64 && k_steps <= 12) ? 64 : 128;
-  if (!a8 && tiles(192) <= sm_count && k_steps <= 24) return 192;
-  const int64_t waves = (tiles(256) + sm_count - 1) / sm_count;
-  return (mt & 1) != 0 && tiles(256) * 100 >= waves * sm_count * 97 ? 256 : 0;
+  auto waves = [&](int bn) { return (tiles(bn) + sms - 1) / sms; };
+  auto fills = [&](int bn, int percent) { return tiles(bn) * 100 >= waves(bn) * sms * percent; };
+  if (tiles(128) <= sms) return (!a8 && tiles(128) * 2 <= sms && m > 64 && k_steps <= 12) ? 64 : 128;
+  if (!a8) {
+    if (k_steps <= 3 || (k_steps == 4 && tiles(192) <= 10 * sms)) return tiles(192) > 4 * sms ? 192 : 128;
+    if (k_steps <= 24 && tiles(192) <= sms) return 192;
+    if (k_steps <= 24 && tiles(256) <= sms && fills(256, 80)) return 256;
+    if (k_steps <= 12 && waves(192) <= 3 && fills(192, 90)) return 192;
+  }
+  return mt == 3 && k_steps <= 24 && fills(256, 97) ? 256 : 0;
 }
 
 std::atomic<int> g_force_gemm_kernel{0};  // tuning hook: 0 = automatic, 1 = one CTA per tile, 2 = CTA pairs (two accumulators), 3 = CTA pairs (wide tiles)

@@ -9,8 +9,12 @@ pytestmark = pytest.mark.gpu
                                    (300, 200, 4096),      # the same with long K: 128-wide, a part-filled column
                                    (385, 4736, 256),      # 37 x 4 tiles of 128: a wave to the last SM
                                    (385, 4744, 256),      # one column more: 192-wide
+                                   (1000, 4100, 1024),    # four K-steps, two waves: 128-wide
+                                   (2100, 12288, 256),    # one K-step, seven waves: 192-wide
                                    (512, 7104, 6144),     # 24 K-steps, the last with 192-wide tiles
-                                   (333, 37888, 256)])    # three row tiles, three full waves of 256-wide ones
+                                   (600, 7168, 1280),     # most of a wave of 256-wide tiles
+                                   (600, 10240, 1280),    # two nearly full waves of 192-wide ones
+                                   (333, 37888, 1280)])   # three row tiles, three full waves of 256-wide ones
 @pytest.mark.parametrize("a8", [False, True], ids=["mxfp4", "mxfp8"])
 def test_same_bits_as_the_pairs(batq, S, M, N, a8):
     """Every kernel adds the K-steps of an output in the same order, so the choice changes no bit (rows quantised
