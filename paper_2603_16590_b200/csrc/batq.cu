@@ -63,7 +63,7 @@ struct batq_weight {
   CUtensorMap tmap_b32;   // boxes of 32 weight rows: the CTA-pair kernel composes its half tiles from them
   CUtensorMap tmap_sf;    // scale atoms: [row tiles x KA] rows of 512 bytes, boxes of two atoms
   // CTA-pair schedules already worked out for this weight, by token count (host only)
-  struct SchedEntry { int64_t s; int force_bn; bool wide, a8; double cost; int32_t n_cols, n_segs, pairs; batq::PairSeg seg[batq::kPairMaxSegs]; };
+  struct SchedEntry { int64_t s; int force_bn; bool wide, a8; double cost, cost8; int32_t n_cols, n_segs, pairs; batq::PairSeg seg[batq::kPairMaxSegs]; };
   mutable std::mutex sched_mutex;
   mutable std::vector<SchedEntry> sched_cache;
   bool has_u4;            // n % 128 == 0: the maps below exist (W4A8 GEMM)
@@ -822,18 +822,21 @@ bool pair_schedule(int64_t s, int64_t m, int64_t k_steps, int sm_count, PairPara
 // 0.17 + 0.0009 bn us (0.40 at 256, 0.52 at 384: the bytes the SM pulls from L2), one of a 448-wide
 // tile 0.66 us (four stages of 49 KiB turn over at the latency of a load from L2); about 1.4 us
 // per tile pass between the last MMA of one tile and the first of the next.
-// With MXFP8 activations (a8) the tensor cores run at half the rate and are the only limit:
-// 0.60 us per 256 elements of K at 256 columns, in proportion to the width.
+// With MXFP8 activations (a8): fitted to every forced width of either kernel on 5 layers of 2048 to 13824 channels
+// at 512, 1024 and 2048 tokens (rms 3.5 %).
 double wide_tile_us(int bn, int64_t k_steps, bool a8 = false) {
-  const double step = a8 ? 0.60 * bn / 256.0 : (bn > 384 ? 0.66 : 0.17 + 0.0009 * bn);
-  return static_cast<double>(k_steps) * step + 1.4;
+  const double step8 = bn <= 192 ? 0.487 : bn <= 256 ? 0.517 : bn <= 320 ? 0.652 : bn <= 384 ? 0.692 : 0.795;
+  const double step = a8 ? step8 : (bn > 384 ? 0.66 : 0.17 + 0.0009 * bn);
+  return static_cast<double>(k_steps) * step + (a8 ? 0.8 : 1.4);
 }
 // The same for the two-accumulator kernel: bound by its loads (36 KiB per K-step at 256 columns),
 // the epilogue hidden unless two tiles in a row need the same accumulator.
-double pair_tile_us(int bn, int64_t k_steps, bool same_slot) {
+double pair_tile_us(int bn, int64_t k_steps, bool same_slot, bool a8 = false) {
+  if (a8) return static_cast<double>(k_steps) * (bn <= 192 ? 0.426 : 0.498) + (same_slot ? 0.5 : 0.0);
   return static_cast<double>(k_steps) * 0.383 * (32.0 + bn / 8.0) / 64.0 + (same_slot ? 1.7 : 1.1);
 }
 
+constexpr double kPairFixedUs = 1.5;
 constexpr double kWideFixedUs = 5.5;   // launch, first loads, the last tile's stores
 double wide_cost(const PairSched& c, PairParams* p, int64_t k_steps, int max_pairs, bool a8, double limit, int* pairs_out) {
   p->n_cols = c.n_cols;
@@ -854,7 +857,7 @@ double wide_cost(const PairSched& c, PairParams* p, int64_t k_steps, int max_pai
 }
 
 // The two-accumulator schedule's cost in the same unit, for the choice between the kernels.
-double pair_cost_us(PairParams* p, int64_t k_steps, int np) {
+double pair_cost_us(PairParams* p, int64_t k_steps, int np, bool a8 = false) {
   double worst = 0.0;
   for (int pr = 0; pr < np; ++pr) {
     PairWalk walk(*p, pr, np);
@@ -866,12 +869,12 @@ double pair_cost_us(PairParams* p, int64_t k_steps, int np) {
       int slot;
       uint32_t phase;
       slots.take(t.bn, slot, phase);
-      cost += pair_tile_us(t.bn, k_steps, slot == last);
+      cost += pair_tile_us(t.bn, k_steps, slot == last, a8);
       last = slot;
     }
     worst = std::max(worst, cost);
   }
-  return worst + 1.5;   // the last tile's epilogue
+  return worst + kPairFixedUs;   // the last tile's epilogue
 }
 
 bool wide_schedule(int64_t s, int64_t m, int64_t k_steps, int sm_count, int force_w, bool a8, PairParams* p, int* pairs,
@@ -932,7 +935,8 @@ bool wide_schedule(int64_t s, int64_t m, int64_t k_steps, int sm_count, int forc
 // candidates; a layer is called with few distinct token counts).
 bool pair_schedule_cached(const batq_weight* w, int64_t s, int sm_count, bool wide, PairParams* p, int* pairs,
                           double* cost_us, bool a8 = false) {
-  a8 = a8 && wide;   // the activations' format only enters the wide tiles' cost
+  const bool want8 = a8;
+  a8 = a8 && wide;   // the two-accumulator schedule is the same for either format, only its cost differs
   const int force_bn = g_force_bn.load(std::memory_order_relaxed);
   {
     std::lock_guard<std::mutex> lock(w->sched_mutex);
@@ -945,7 +949,7 @@ bool pair_schedule_cached(const batq_weight* w, int64_t s, int sm_count, bool wi
         p->n_segs = e.n_segs;
         for (int i = 0; i < kPairMaxSegs; ++i) p->seg[i] = e.seg[i];
         *pairs = e.pairs;
-        *cost_us = e.cost;
+        *cost_us = want8 ? e.cost8 : e.cost;
         return true;
       }
   }
@@ -957,10 +961,12 @@ bool pair_schedule_cached(const batq_weight* w, int64_t s, int sm_count, bool wi
     if (!pair_schedule(s, w->m, k_steps, sm_count, p, pairs)) return false;
     *cost_us = pair_cost_us(p, k_steps, *pairs);
   }
+  const double cost8 = wide ? *cost_us : pair_cost_us(p, k_steps, *pairs, true);
   batq_weight::SchedEntry e{};
-  e.s = s; e.force_bn = force_bn; e.wide = wide; e.a8 = a8; e.cost = *cost_us;
+  e.s = s; e.force_bn = force_bn; e.wide = wide; e.a8 = a8; e.cost = *cost_us; e.cost8 = cost8;
   e.n_cols = p->n_cols; e.n_segs = p->n_segs; e.pairs = *pairs;
   for (int i = 0; i < kPairMaxSegs; ++i) e.seg[i] = p->seg[i];
+  *cost_us = want8 ? cost8 : e.cost;
   std::lock_guard<std::mutex> lock(w->sched_mutex);
   if (w->sched_cache.size() >= 16) w->sched_cache.erase(w->sched_cache.begin());
   w->sched_cache.push_back(e);
@@ -1490,9 +1496,7 @@ batq_status launch_gemm_w4a8(const void* x_codes8, const void* x_sf, const batq_
   if (st != BATQ_OK) return st;
   // CTA pairs above 128 tokens (two 128-token tiles to share a weight tile), as in the W4A4 GEMM:
   // tiles of up to 256 features on two accumulators, or tiles of up to 448 on one.  kind::mxf8f6f4
-  // runs at half the rate of kind::mxf4, so the wide tile (fewer bytes per flop, tensor-bound) is
-  // the rule here; the two-accumulator kernel keeps the layers where a pair has at most two tiles
-  // whichever way the features are cut.
+  // runs at half the rate of kind::mxf4; the cost model with that format's constants decides.
   const int force_gemm = g_force_gemm_kernel.load(std::memory_order_relaxed);
   const bool free_choice = force_gemm == 0 && s > 128 && w->m >= 192;
   const int cta_bn = free_choice && g_force_bn.load(std::memory_order_relaxed) == 0
@@ -1513,20 +1517,11 @@ batq_status launch_gemm_w4a8(const void* x_codes8, const void* x_sf, const batq_
       if (!pair_schedule_cached(w, s, info->sm_count, true, &pw, &pairs_w, &us_w, true)) return BATQ_ERR_SHAPE;
       wide = true;
     } else {
-      if (!pair_schedule_cached(w, s, info->sm_count, false, &p, &pairs, &us)) return BATQ_ERR_SHAPE;
+      if (!pair_schedule_cached(w, s, info->sm_count, false, &p, &pairs, &us, true)) return BATQ_ERR_SHAPE;
       if (force_gemm == 0 && force_bn == 0 && w->m >= 320 &&
           pair_schedule_cached(w, s, info->sm_count, true, &pw, &pairs_w, &us_w, true)) {
-        // four or more tiles for some pair in the two-accumulator schedule: take the wide tiles
-        // (measured at 2048 tokens: gate/up, 14 tiles, 158 against 172 us; qkv, 3 tiles, 39.5 against 37.3)
-        int max_tiles = 0;
-        for (int pr = 0; pr < pairs; ++pr) {
-          PairWalk walk(p, pr, pairs);
-          PairTile t;
-          int cnt = 0;
-          while (walk.next(t)) ++cnt;
-          max_tiles = std::max(max_tiles, cnt);
-        }
-        wide = max_tiles >= 4;
+        // The fit's constants: a wide schedule's first tile has no accumulator to wait for.
+        wide = us_w - kWideFixedUs - 0.8 < us - kPairFixedUs;
       }
     }
     if (wide) {
