@@ -607,6 +607,15 @@ batq_status make_y_tmap(CUtensorMap* map, const void* base, int64_t rows, int64_
   return r == CUDA_SUCCESS ? BATQ_OK : BATQ_ERR_CUDA;
 }
 
+// Below half a wave of 128-wide tiles: twice as many 64-wide ones where K is short (a few dozen CTAs cannot pull the
+// weights fast enough, a CTA streams what its ring keeps in flight), not where the activation tile, loaded by
+// twice as many CTAs, has many K-steps.  Whole layers of 64, 100 and 128 tokens, 64- / 128-wide: 1024 -> 1024 5.1 / 5.5 us,
+// 2048 -> 2048 6.3 / 6.8, 3072 -> 3072 8.3 / 8.7, 4096 -> 1024 8.7 / 9.0 (8 tiles), but 3584 -> 4608 9.5 / 9.0, 4096 -> 4096 9.93 / 9.84, 4096 ->
+// 8192 10.9 / 10.5, 5120 -> 5120 11.5 / 11.1, 8192 -> 1024 14.6 / 14.0.
+inline bool narrow_tiles_pay(int64_t tiles128, int64_t k_steps, int sm_count) {
+  return tiles128 * 2 <= sm_count && (k_steps <= 12 || (k_steps <= 16 && tiles128 * 8 <= sm_count));
+}
+
 // Tile width.  192 and 128 keep two accumulators in tensor memory (the epilogue of a tile
 // overlaps the main loop of the next); 256 has the highest flop per byte staged but a single
 // accumulator.  Pick by modelled time: waves x (main loop + exposed epilogue), with the main
@@ -616,9 +625,8 @@ int pick_bn(int64_t s, int64_t m, int64_t n, int sm_count) {
   const int force_bn = g_force_bn.load(std::memory_order_relaxed);
   if (force_bn == 64 || force_bn == 128 || force_bn == 192 || force_bn == 256) return force_bn;
   const int64_t mt = (s + kBM - 1) / kBM;
-  // A few dozen tiles cannot pull the weights fast enough (a CTA streams what its ring keeps in
-  // flight): below half a wave of 128-wide tiles, twice as many 64-wide ones.
-  if (mt * ((m + 127) / 128) * 2 <= sm_count && m > 64) return 64;
+  if (narrow_tiles_pay(mt * ((m + 127) / 128), (n + 255) / 256, sm_count) && m > 64) return 64;
+  if (mt * ((m + 127) / 128) * 2 <= sm_count) return 128;
   const double k_steps = static_cast<double>((n + 255) / 256);
   auto cost = [&](int bn, double exposed_epilogue) {
     const int64_t tiles = mt * ((m + bn - 1) / bn);
@@ -656,7 +664,7 @@ int one_cta_width(int64_t s, int64_t m, int64_t n, int sm_count, bool a8) {
   auto tiles = [&](int bn) { return mt * ((m + bn - 1) / bn); };
   auto waves = [&](int bn) { return (tiles(bn) + sms - 1) / sms; };
   auto fills = [&](int bn, int percent) { return tiles(bn) * 100 >= waves(bn) * sms * percent; };
-  if (tiles(128) <= sms) return (!a8 && tiles(128) * 2 <= sms && m > 64 && k_steps <= 12) ? 64 : 128;
+  if (tiles(128) <= sms) return (!a8 && m > 64 && narrow_tiles_pay(tiles(128), k_steps, sm_count)) ? 64 : 128;
   if (!a8) {
     if (k_steps <= 3 || (k_steps == 4 && tiles(192) <= 10 * sms)) return tiles(192) > 4 * sms ? 192 : 128;
     if (k_steps <= 24 && tiles(192) <= sms) return 192;

@@ -1,4 +1,4 @@
-"""Above 128 tokens: the layers that one CTA per 128-token tile takes instead of the CTA pairs.  GPU only."""
+"""The layers that one CTA per 128-token tile takes, above 128 tokens instead of the CTA pairs.  GPU only."""
 import pytest
 import torch
 
@@ -7,6 +7,8 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("S,M,N", [(129, 1024, 512),      # half a wave of 128-wide tiles, short K: 64-wide
                                    (300, 200, 4096),      # the same with long K: 128-wide, a part-filled column
+                                   (100, 4616, 3584),     # up to 128 tokens: long K, 128-wide though half a wave
+                                   (128, 1024, 4096),     # 16 K-steps and few tiles: 64-wide
                                    (385, 4736, 256),      # 37 x 4 tiles of 128: a wave to the last SM
                                    (385, 4744, 256),      # one column more: 192-wide
                                    (1000, 4100, 1024),    # four K-steps, two waves: 128-wide
