@@ -359,8 +359,11 @@ quantize_act_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_
       }
       const int pb = (n_img - 1) & 1;
       const int buf = it % kQtDBufs;
-      ok = __all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&d_empty[buf]), (static_cast<uint32_t>(it / kQtDBufs) & 1u) ^ 1u, &abort_flag));
-      if (!ok) break;
+      if (it >= kQtABufs) {   // the MMAs of the unit whose X is about to be overwritten
+        const int old = it - kQtABufs;
+        ok = __all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&d_full[old % kQtDBufs]), static_cast<uint32_t>(old / kQtDBufs) & 1u, &abort_flag));
+        if (!ok) break;
+      }
       ok = __all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&x_full[stage]), phase, &abort_flag));
       if (!ok) break;
       tc_fence_after_sync();
@@ -368,14 +371,20 @@ quantize_act_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_
       const uint64_t a_stage = a_desc0 + static_cast<uint32_t>((stage * kQtStageBytes) >> 4);
       const uint64_t b_img = b_desc0 + static_cast<uint32_t>((pb * kQtStripImageBytes) >> 4);
       const uint32_t d0 = tmem_base + buf * (kQtGroups * 32);
-      const uint32_t a_tmem = tmem_base + kQtDBufs * (kQtGroups * 32) + (it & 1) * kQtACols;
+      const uint32_t a_tmem = tmem_base + kQtDBufs * (kQtGroups * 32) + (it % kQtABufs) * kQtACols;
       if (elect_one()) {
-        // X into tensor memory first, 16 channels (32 bytes a row) at a time; cp and mma of one thread
-        // execute in issue order.
+        // X into tensor memory first, 16 channels (32 bytes a row) at a time.  PTX has a copy and the MMAs that one
+        // thread issues behind it execute in that order; the other way round it promises nothing, hence the wait above.
 #pragma unroll
         for (int c = 0; c < 2 * kQtGroups; ++c)   // channels 16 c .. 16 c + 15: box c / 4, byte offset (c % 4) * 32 of its rows
           tc_cp_128x256b(a_tmem + 8 * c, a_stage + static_cast<uint32_t>(((c >> 2) * kQtBoxBytes + (c & 3) * 32) >> 4));
         tc_commit(smem_u32(&x_empty[stage]));
+      }
+      __syncwarp();
+      ok = __all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&d_empty[buf]), (static_cast<uint32_t>(it / kQtDBufs) & 1u) ^ 1u, &abort_flag));
+      if (!ok) break;
+      tc_fence_after_sync();
+      if (elect_one()) {
 #pragma unroll
         for (int g = 0; g < kQtGroups; ++g) {
           if (g < ng) {

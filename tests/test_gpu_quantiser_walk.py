@@ -42,3 +42,37 @@ def test_every_unit_is_quantised_once(batq, S, N, fp8):
     finally:
         batq.batq_debug_force_quantizer(0)
     assert batq.batq_last_device_status() == 0
+
+
+@pytest.mark.parametrize("units", [1, 2, 3, 4, 5, 7, 13])
+@pytest.mark.parametrize("fp8", [False, True], ids=["mxfp4", "mxfp8"])
+def test_buffers_are_reused_in_turn(batq, units, fp8):
+    """`units` units for every CTA but the last ones, around the counts of its buffers in tensor memory (two of X, three
+    of accumulators), of input stages (three) and of staging tiles (four).  Units differ in magnitude, and
+    the reference quantises one unit a CTA, which reuses no buffer: whole numbers, no tolerance."""
+    n, sms = 128, torch.cuda.get_device_properties(0).multi_processor_count
+    s = 128 * sms * units - 3
+    t = synth.make_transform(n, 7, "baseline")
+    tr = batq.batq_transform_create(n, t.left, t.right, t.clip_lo, t.clip_hi)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(units)
+    x = torch.randn((s, n), generator=gen, device="cuda")
+    tile = torch.arange(s, device="cuda") // 128
+    x = (x * torch.exp2((tile * 7 % 11 - 5).float())[:, None]).to(torch.bfloat16)
+    fn = batq.batq_quantize_act_mxfp8 if fp8 else batq.batq_quantize_act
+
+    def run(rows):
+        codes = torch.zeros((rows.shape[0], n if fp8 else n // 2), dtype=torch.uint8, device="cuda")
+        scales = torch.zeros((rows.shape[0], n // 32), dtype=torch.uint8, device="cuda")
+        fn(tr, rows, codes, scales, batq.SF_ROWMAJOR)
+        return codes, scales
+
+    batq.batq_debug_force_quantizer(2)
+    try:
+        whole = run(x)
+        parts = [run(p) for p in x.split(128 * sms)]
+    finally:
+        batq.batq_debug_force_quantizer(0)
+    assert batq.batq_last_device_status() == 0
+    for got, want in zip(whole, zip(*parts)):
+        assert torch.equal(got, torch.cat(want))
