@@ -39,6 +39,12 @@ int32_t batq_debug_pair_schedule(int64_t s, int64_t m, int64_t n, int32_t sm_cou
 int32_t batq_debug_wide_schedule(int64_t s, int64_t m, int64_t n, int32_t sm_count, int32_t pair,
                                  int32_t* tiles, int32_t max_tiles);
 
+/* Host only, no GPU needed: the kernel that batq_gemm_mxfp4 (mxfp8 != 0: batq_gemm_mxfp8_mxfp4) takes for an s x m output
+ * over n input channels on a device with sm_count SMs, counted as in batq_debug_force_gemm_kernel: 1 = one CTA per 128-token
+ * tile, 2 = CTA pairs with two accumulators, 3 = CTA pairs with wide tiles, 4 = the swapped-operand kernel.  *width
+ * (may be NULL) receives the width of its first column of tiles in features.  -1 for arguments out of range. */
+int32_t batq_debug_gemm_choice(int64_t s, int64_t m, int64_t n, int32_t sm_count, int32_t mxfp8, int32_t* width);
+
 /* Which prefill GEMM kernel later calls use.  0 = automatic (up to 128 tokens, and where the device
  * has an SM for every tile at once or an odd number of row tiles fills its waves, one CTA per
  * 128-token tile; else CTA pairs sharing a 256-token tile, with tiles of up to 256 features and two

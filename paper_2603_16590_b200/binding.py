@@ -59,6 +59,7 @@ SIGNATURES = {
     "batq_linear_kernel_launches": (C.c_int32, [_P, _P, _I64]),
     "batq_debug_pair_schedule": (C.c_int32, [_I64, _I64, _I64, _I32, _I32, _P, _I32]),
     "batq_debug_wide_schedule": (C.c_int32, [_I64, _I64, _I64, _I32, _I32, _P, _I32]),
+    "batq_debug_gemm_choice": (C.c_int32, [_I64, _I64, _I64, _I32, _I32, C.POINTER(_I32)]),
     "batq_linear_w4a4": (C.c_int, [_P, _P, _P, _I64, _I64, _P, _I32, _I64, _P, _SZ, _P]),
     "batq_linear_w4a4_host": (C.c_int, [_P, _P, _P, _I64, _P, _I32, _P, _P, _P, _SZ, _P]),
     "batq_linear_w4a4_host_async": (C.c_int, [_P, _P, _P, _I64, _P, _I32, _P, _P, _P, _SZ, _P]),
@@ -365,6 +366,15 @@ def batq_debug_pair_schedule(s, m, n, sm_count=148):
 def batq_debug_wide_schedule(s, m, n, sm_count=148):
     """The same for the wide-tile CTA-pair GEMM (host only)."""
     return _schedule(load().batq_debug_wide_schedule, s, m, n, sm_count)
+
+
+def batq_debug_gemm_choice(s, m, n, mxfp8=False, sm_count=148):
+    """(kernel, width of its first column of tiles) of a GEMM call (host only)."""
+    width = _I32(0)
+    kernel = load().batq_debug_gemm_choice(s, m, n, sm_count, 1 if mxfp8 else 0, C.byref(width))
+    if kernel < 0:
+        raise ValueError("bad shape")
+    return kernel, width.value
 
 
 def batq_linear_kernel_launches(t, w: Weight, s) -> int:

@@ -10,6 +10,7 @@
 #include <climits>
 #include <cmath>
 #include <cstring>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <vector>
@@ -830,8 +831,8 @@ bool pair_schedule(int64_t s, int64_t m, int64_t k_steps, int sm_count, PairPara
 // 0.17 + 0.0009 bn us (0.40 at 256, 0.52 at 384: the bytes the SM pulls from L2), one of a 448-wide
 // tile 0.66 us (four stages of 49 KiB turn over at the latency of a load from L2); about 1.4 us
 // per tile pass between the last MMA of one tile and the first of the next.
-// With MXFP8 activations (a8): fitted to every forced width of either kernel on 5 layers of 2048 to 13824 channels
-// at 512, 1024 and 2048 tokens (rms 3.5 %).
+// With MXFP8 activations (a8), for the choice among schedules of this kernel alone: fitted to its forced widths on 5
+// layers of 2048 to 13824 channels at 512, 1024 and 2048 tokens.
 double wide_tile_us(int bn, int64_t k_steps, bool a8 = false) {
   const double step8 = bn <= 192 ? 0.487 : bn <= 256 ? 0.517 : bn <= 320 ? 0.652 : bn <= 384 ? 0.692 : 0.795;
   const double step = a8 ? step8 : (bn > 384 ? 0.66 : 0.17 + 0.0009 * bn);
@@ -839,12 +840,10 @@ double wide_tile_us(int bn, int64_t k_steps, bool a8 = false) {
 }
 // The same for the two-accumulator kernel: bound by its loads (36 KiB per K-step at 256 columns),
 // the epilogue hidden unless two tiles in a row need the same accumulator.
-double pair_tile_us(int bn, int64_t k_steps, bool same_slot, bool a8 = false) {
-  if (a8) return static_cast<double>(k_steps) * (bn <= 192 ? 0.426 : 0.498) + (same_slot ? 0.5 : 0.0);
+double pair_tile_us(int bn, int64_t k_steps, bool same_slot) {
   return static_cast<double>(k_steps) * 0.383 * (32.0 + bn / 8.0) / 64.0 + (same_slot ? 1.7 : 1.1);
 }
 
-constexpr double kPairFixedUs = 1.5;
 constexpr double kWideFixedUs = 5.5;   // launch, first loads, the last tile's stores
 double wide_cost(const PairSched& c, PairParams* p, int64_t k_steps, int max_pairs, bool a8, double limit, int* pairs_out) {
   p->n_cols = c.n_cols;
@@ -865,7 +864,7 @@ double wide_cost(const PairSched& c, PairParams* p, int64_t k_steps, int max_pai
 }
 
 // The two-accumulator schedule's cost in the same unit, for the choice between the kernels.
-double pair_cost_us(PairParams* p, int64_t k_steps, int np, bool a8 = false) {
+double pair_cost_us(PairParams* p, int64_t k_steps, int np) {
   double worst = 0.0;
   for (int pr = 0; pr < np; ++pr) {
     PairWalk walk(*p, pr, np);
@@ -877,12 +876,44 @@ double pair_cost_us(PairParams* p, int64_t k_steps, int np, bool a8 = false) {
       int slot;
       uint32_t phase;
       slots.take(t.bn, slot, phase);
-      cost += pair_tile_us(t.bn, k_steps, slot == last, a8);
+      cost += pair_tile_us(t.bn, k_steps, slot == last);
       last = slot;
     }
     worst = std::max(worst, cost);
   }
-  return worst + kPairFixedUs;   // the last tile's epilogue
+  return worst + 1.5;   // the last tile's epilogue
+}
+
+// The choice between the kernels with MXFP8 activations: when the last pair is done with its tiles, in microseconds after
+// the first MMA.  The MMAs of a tile start once those of the tile before it and the read-out of its accumulator have
+// ended; a read-out starts behind the tile's MMAs and the read-out (wide tiles: and the stores) of the tile before.  Step,
+// read-out and store times are fitted to 228 layers (19 widths of 512 to 18944 channels and 3072 to 37888 features, at 12
+// counts of 129 to 3000 tokens), each with every forced width of either kernel and with both schedules, replayed in turn in
+// one process: rms 2.4 %.  The choice by these times is 0.1 % behind the better kernel on average and 4 % at worst
+// (1024 -> 8192 at 1500 tokens); with tile times added up and the wide kernel's fixed cost left out it was 0.5 % and
+// 19 % (512 -> 16384 at 3000 tokens, pairs 42.8 us, wide 35.9; 1024 -> 8192 at 1024, 15.4 and 16.8), and with the
+// wide kernel from four tiles a pair on 1.1 % and 20 % (13824 -> 5120 at 896, 73.9 and 61.7).
+double a8_cost_us(const PairParams& p, int64_t k_steps, int np, bool wide) {
+  double worst = 0.0;
+  for (int pr = 0; pr < np; ++pr) {
+    PairWalk walk(p, pr, np);
+    PairSlots slots;
+    PairTile t;
+    double mma_end = 0.0, out_end = 0.0, free_at[2] = {0.0, 0.0};
+    while (walk.next(t)) {
+      const int bn = t.bn;
+      int slot = 0;
+      uint32_t phase;
+      if (!wide) slots.take(bn, slot, phase);
+      const double step = !wide ? (bn <= 64 ? 0.38 : bn <= 128 ? 0.47 : bn <= 192 ? 0.49 : 0.54)
+                                : (bn <= 128 ? 0.53 : bn <= 192 ? 0.56 : bn <= 256 ? 0.60 : bn <= 320 ? 0.735 : bn <= 384 ? 0.815 : 0.95);
+      mma_end = std::max(mma_end, free_at[slot]) + static_cast<double>(k_steps) * step;
+      free_at[slot] = std::max(mma_end, out_end) + (wide ? 0.72 : 1.05 + 0.4 * bn / 256.0);
+      out_end = free_at[slot] + (wide ? 1.1 * bn / 256.0 : 0.0);
+    }
+    worst = std::max(worst, out_end);
+  }
+  return worst;
 }
 
 bool wide_schedule(int64_t s, int64_t m, int64_t k_steps, int sm_count, int force_w, bool a8, PairParams* p, int* pairs,
@@ -969,7 +1000,7 @@ bool pair_schedule_cached(const batq_weight* w, int64_t s, int sm_count, bool wi
     if (!pair_schedule(s, w->m, k_steps, sm_count, p, pairs)) return false;
     *cost_us = pair_cost_us(p, k_steps, *pairs);
   }
-  const double cost8 = wide ? *cost_us : pair_cost_us(p, k_steps, *pairs, true);
+  const double cost8 = a8_cost_us(*p, k_steps, *pairs, wide);
   batq_weight::SchedEntry e{};
   e.s = s; e.force_bn = force_bn; e.wide = wide; e.a8 = a8; e.cost = *cost_us; e.cost8 = cost8;
   e.n_cols = p->n_cols; e.n_segs = p->n_segs; e.pairs = *pairs;
@@ -979,6 +1010,58 @@ bool pair_schedule_cached(const batq_weight* w, int64_t s, int sm_count, bool wi
   if (w->sched_cache.size() >= 16) w->sched_cache.erase(w->sched_cache.begin());
   w->sched_cache.push_back(e);
   return true;
+}
+
+// The kernel of a GEMM call, counted as in batq_debug_force_gemm_kernel; kSwappedGemm: the swapped-operand one.
+enum GemmKernel { kOneCtaGemm = 1, kPairGemm = 2, kWideGemm = 3, kSwappedGemm = 4 };
+
+// One CTA per 128-token tile, and how wide its tiles are, or CTA pairs.
+bool one_cta_gemm(const batq_weight* w, int64_t s, int sm_count, bool a8, int* bn) {
+  const int force_gemm = g_force_gemm_kernel.load(std::memory_order_relaxed);
+  const int force_bn = g_force_bn.load(std::memory_order_relaxed);
+  // CTA pairs need at least two 128-token tiles to pay, and wide enough a layer for their tiles.
+  const bool free_choice = force_gemm == 0 && s > 128 && w->m >= 192;
+  const int cta_bn = free_choice && force_bn == 0 ? one_cta_width(s, w->m, w->n, sm_count, a8) : 0;
+  if (force_gemm == 2 || force_gemm == 3 || (free_choice && cta_bn == 0)) return false;
+  if (cta_bn != 0) {
+    *bn = cta_bn;
+  } else if (!a8) {
+    *bn = pick_bn(s, w->m, w->n, sm_count);
+  } else {
+    // 256 (half the operand bytes per flop of a 128-wide tile; measured 16 % faster on layers of 4096 / 14336
+    // channels at 2048 tokens at equal wave counts) unless 128-wide tiles need clearly fewer waves' worth of time (a
+    // layer too small to fill the SMs with 256-wide tiles).
+    const int64_t mt = (s + kBM - 1) / kBM;
+    auto waves = [&](int wd) { return ((mt * ((w->m + wd - 1) / wd)) + sm_count - 1) / sm_count; };
+    *bn = (w->m <= 128 || waves(128) * 128 * 1.2 < waves(256) * 256) ? 128 : 256;
+    if (force_bn == 128 || force_bn == 256) *bn = force_bn;
+  }
+  return true;
+}
+
+// Which of the two pair kernels: tiles of up to 256 features on two accumulators, or of up to 448 on one; each comes with
+// its own schedule and an estimate of its time.
+batq_status pick_pair_kernel(const batq_weight* w, int64_t s, int sm_count, bool a8, PairParams* p, int* pairs, bool* wide) {
+  const int force_gemm = g_force_gemm_kernel.load(std::memory_order_relaxed);
+  const int force_bn = g_force_bn.load(std::memory_order_relaxed);
+  const bool wide_width = force_bn == 0 || (force_bn >= 64 && force_bn <= kWideMaxBn && force_bn % 64 == 0);
+  if (a8 && force_gemm == 3 && !wide_width) return BATQ_ERR_SHAPE;
+  double us = 0.0, us_w = 0.0;
+  if (force_gemm == 3 && wide_width) {
+    *wide = true;
+    return pair_schedule_cached(w, s, sm_count, true, p, pairs, &us_w, a8) ? BATQ_OK : BATQ_ERR_SHAPE;
+  }
+  *wide = false;
+  if (!pair_schedule_cached(w, s, sm_count, false, p, pairs, &us, a8)) return BATQ_ERR_SHAPE;
+  PairParams pw{};
+  int pairs_w = 0;
+  if (force_gemm == 0 && force_bn == 0 && w->m >= 320 && pair_schedule_cached(w, s, sm_count, true, &pw, &pairs_w, &us_w, a8) &&
+      us_w < us) {
+    *wide = true;
+    *p = pw;
+    *pairs = pairs_w;
+  }
+  return BATQ_OK;
 }
 
 template <bool BF, bool WIDE>
@@ -1010,34 +1093,16 @@ batq_status launch_gemm_pair(const void* x_codes, const void* x_sf, const batq_w
   CUtensorMap tmap_sfa;
   batq_status st = make_sf_tmap(&tmap_sfa, x_sf, (s + 127) / 128, w->katoms);
   if (st != BATQ_OK) return st;
-  // Two kernels share this launcher: tiles of up to 256 features with two accumulators, or tiles of
-  // up to 448 with one; each comes with its own schedule and an estimate of its time.
-  const int force_gemm = g_force_gemm_kernel.load(std::memory_order_relaxed);
-  const int force_bn = g_force_bn.load(std::memory_order_relaxed);
-  const bool may_wide = force_gemm == 3 ? (force_bn == 0 || (force_bn >= 64 && force_bn <= kWideMaxBn && force_bn % 64 == 0))
-                                        : (w->m >= 320 && force_bn == 0);
-  PairParams p{}, pw{};
-  int pairs = 0, pairs_w = 0;
-  double us = 0.0, us_w = 0.0;
+  PairParams p{};
+  int pairs = 0;
   bool wide = false;
-  if (force_gemm == 3 && may_wide) {
-    if (!pair_schedule_cached(w, s, sm_count, true, &pw, &pairs_w, &us_w)) return BATQ_ERR_SHAPE;
-    wide = true;
-  } else {
-    if (!pair_schedule_cached(w, s, sm_count, false, &p, &pairs, &us)) return BATQ_ERR_SHAPE;
-    if (force_gemm == 0 && may_wide &&
-        pair_schedule_cached(w, s, sm_count, true, &pw, &pairs_w, &us_w))
-      wide = us_w < us;
-  }
+  st = pick_pair_kernel(w, s, sm_count, false, &p, &pairs, &wide);
+  if (st != BATQ_OK) return st;
   CUtensorMap tmap_y64;
   std::memset(&tmap_y64, 0, sizeof(tmap_y64));
-  if (wide) {
-    p = pw;
-    pairs = pairs_w;
-    if (m16 > 0) {   // the wide kernel stages its output in boxes of 64-byte rows
-      st = make_y_tmap(&tmap_y64, y, s, m16, ldy, bf, 64);
-      if (st != BATQ_OK) return st;
-    }
+  if (wide && m16 > 0) {   // the wide kernel stages its output in boxes of 64-byte rows
+    st = make_y_tmap(&tmap_y64, y, s, m16, ldy, bf, 64);
+    if (st != BATQ_OK) return st;
   }
   p.katoms = w->katoms;
   p.k_steps = static_cast<int32_t>((w->n + 255) / 256);
@@ -1070,14 +1135,9 @@ batq_status launch_gemm(const void* x_codes, const void* x_sf, const batq_weight
   const int64_t m16 = w->m / (bf ? 8 : 4) * (bf ? 8 : 4);
   if (st == BATQ_OK && m16 > 0) st = make_y_tmap(&tmap_y, y, s, m16, ldy, bf);
   if (st != BATQ_OK) return st;
-  // CTA pairs need at least two 128-token tiles to pay, and wide enough a layer for their tiles.
-  const int force_gemm = g_force_gemm_kernel.load(std::memory_order_relaxed);
-  const bool free_choice = force_gemm == 0 && s > 128 && w->m >= 192;
-  const int cta_bn = free_choice && g_force_bn.load(std::memory_order_relaxed) == 0
-                         ? one_cta_width(s, w->m, w->n, info->sm_count, false) : 0;
-  const bool use_pair = force_gemm == 2 || force_gemm == 3 || (free_choice && cta_bn == 0);
-  if (use_pair) return launch_gemm_pair(x_codes, x_sf, w, s, y, bf, ldy, stream, info->sm_count, tmap_a, tmap_y, m16, dependent);
-  const int bn = cta_bn != 0 ? cta_bn : pick_bn(s, w->m, w->n, info->sm_count);
+  int bn = 0;
+  if (!one_cta_gemm(w, s, info->sm_count, false, &bn))
+    return launch_gemm_pair(x_codes, x_sf, w, s, y, bf, ldy, stream, info->sm_count, tmap_a, tmap_y, m16, dependent);
   GemmParams p{};
   p.sfa = static_cast<const uint8_t*>(x_sf);
   p.sfb = w->scales;
@@ -1502,43 +1562,21 @@ batq_status launch_gemm_w4a8(const void* x_codes8, const void* x_sf, const batq_
   const int64_t m16 = w->m / (bf ? 8 : 4) * (bf ? 8 : 4);
   if (st == BATQ_OK && m16 > 0) st = make_y_tmap(&tmap_y, y, s, m16, ldy, bf);
   if (st != BATQ_OK) return st;
-  // CTA pairs above 128 tokens (two 128-token tiles to share a weight tile), as in the W4A4 GEMM:
-  // tiles of up to 256 features on two accumulators, or tiles of up to 448 on one.  kind::mxf8f6f4
-  // runs at half the rate of kind::mxf4; the cost model with that format's constants decides.
-  const int force_gemm = g_force_gemm_kernel.load(std::memory_order_relaxed);
-  const bool free_choice = force_gemm == 0 && s > 128 && w->m >= 192;
-  const int cta_bn = free_choice && g_force_bn.load(std::memory_order_relaxed) == 0
-                         ? one_cta_width(s, w->m, w->n, info->sm_count, true) : 0;
-  if (force_gemm == 2 || force_gemm == 3 || (free_choice && cta_bn == 0)) {
+  // The kernels are chosen as in the W4A4 GEMM, by this format's times: kind::mxf8f6f4 runs at half the rate of kind::mxf4.
+  int bn = 0;
+  if (!one_cta_gemm(w, s, info->sm_count, true, &bn)) {
     CUtensorMap tmap_sfa, tmap_y64;
     std::memset(&tmap_y64, 0, sizeof(tmap_y64));
     st = make_sf_tmap(&tmap_sfa, x_sf, (s + 127) / 128, w->katoms, 1);
     if (st != BATQ_OK) return st;
-    const int force_bn = g_force_bn.load(std::memory_order_relaxed);
-    const bool forced_w = force_bn >= 64 && force_bn <= kWideMaxBn && force_bn % 64 == 0;
-    PairParams p{}, pw{};
-    int pairs = 0, pairs_w = 0;
-    double us = 0.0, us_w = 0.0;
+    PairParams p{};
+    int pairs = 0;
     bool wide = false;
-    if (force_gemm == 3) {
-      if (force_bn != 0 && !forced_w) return BATQ_ERR_SHAPE;
-      if (!pair_schedule_cached(w, s, info->sm_count, true, &pw, &pairs_w, &us_w, true)) return BATQ_ERR_SHAPE;
-      wide = true;
-    } else {
-      if (!pair_schedule_cached(w, s, info->sm_count, false, &p, &pairs, &us, true)) return BATQ_ERR_SHAPE;
-      if (force_gemm == 0 && force_bn == 0 && w->m >= 320 &&
-          pair_schedule_cached(w, s, info->sm_count, true, &pw, &pairs_w, &us_w, true)) {
-        // The fit's constants: a wide schedule's first tile has no accumulator to wait for.
-        wide = us_w - kWideFixedUs - 0.8 < us - kPairFixedUs;
-      }
-    }
-    if (wide) {
-      p = pw;
-      pairs = pairs_w;
-      if (m16 > 0) {
-        st = make_y_tmap(&tmap_y64, y, s, m16, ldy, bf, 64);
-        if (st != BATQ_OK) return st;
-      }
+    st = pick_pair_kernel(w, s, info->sm_count, true, &p, &pairs, &wide);
+    if (st != BATQ_OK) return st;
+    if (wide && m16 > 0) {
+      st = make_y_tmap(&tmap_y64, y, s, m16, ldy, bf, 64);
+      if (st != BATQ_OK) return st;
     }
     p.katoms = w->katoms;
     p.k_steps = static_cast<int32_t>(w->n / kW4A8KElems);
@@ -1569,15 +1607,6 @@ batq_status launch_gemm_w4a8(const void* x_codes8, const void* x_sf, const batq_
     if (e != cudaSuccess) { cudaGetLastError(); return BATQ_ERR_CUDA; }
     return BATQ_OK;
   }
-  // One CTA per tile.  Tile width: 256 (half the operand bytes per flop of a 128-wide tile; measured 16 % faster on
-  // the config-1 shapes at equal wave counts) unless 128-wide tiles need clearly fewer waves' worth
-  // of time (a layer too small to fill the SMs with 256-wide tiles).
-  const int64_t mt = (s + kBM - 1) / kBM;
-  auto waves = [&](int bn) { return ((mt * ((w->m + bn - 1) / bn)) + info->sm_count - 1) / info->sm_count; };
-  const int force_bn = g_force_bn.load(std::memory_order_relaxed);
-  int bn = (w->m <= 128 || waves(128) * 128 * 1.2 < waves(256) * 256) ? 128 : 256;
-  if (force_bn == 128 || force_bn == 256) bn = force_bn;
-  else if (cta_bn != 0) bn = cta_bn;
   W4A8Params p{};
   p.sfa = static_cast<const uint8_t*>(x_sf);
   p.sfb = w->scales;
@@ -1585,7 +1614,7 @@ batq_status launch_gemm_w4a8(const void* x_codes8, const void* x_sf, const batq_
   p.m = static_cast<int32_t>(w->m);
   p.katoms = w->katoms;
   p.k_steps = static_cast<int32_t>(w->n / kW4A8KElems);
-  p.m_tiles = static_cast<int32_t>(mt);
+  p.m_tiles = static_cast<int32_t>((s + kBM - 1) / kBM);
   p.n_tiles = static_cast<int32_t>((w->m + bn - 1) / bn);
   p.sfb_row_tiles = static_cast<int32_t>((w->m + 127) / 128);
   p.m16 = static_cast<int32_t>(m16);
@@ -2249,6 +2278,29 @@ int32_t batq_debug_wide_schedule(int64_t s, int64_t m, int64_t n, int32_t sm_cou
     ++cnt;
   }
   return cnt;
+}
+int32_t batq_debug_gemm_choice(int64_t s, int64_t m, int64_t n, int32_t sm_count, int32_t mxfp8, int32_t* width) {
+  const bool a8 = mxfp8 != 0;
+  if (s <= 0 || m <= 0 || n <= 0 || n % (a8 ? 128 : 32) != 0 || sm_count < 2) return -1;
+  std::unique_ptr<batq_weight> w(new (std::nothrow) batq_weight());
+  if (w == nullptr) return -1;
+  w->m = m;
+  w->n = n;
+  w->sm_count = sm_count;
+  int bn = 0, pairs = 0;
+  bool wide = false;
+  int32_t kernel = kOneCtaGemm;
+  if (a8 && g_force_gemm_kernel.load(std::memory_order_relaxed) == 0 && s <= kSmallSMax && swapped_operands_pay(w.get(), s, true)) {
+    kernel = kSwappedGemm;
+    bn = 128;
+  } else if (!one_cta_gemm(w.get(), s, sm_count, a8, &bn)) {
+    PairParams p{};
+    if (pick_pair_kernel(w.get(), s, sm_count, a8, &p, &pairs, &wide) != BATQ_OK) return -1;
+    kernel = wide ? kWideGemm : kPairGemm;
+    bn = p.seg[0].wa;
+  }
+  if (width != nullptr) *width = bn;
+  return kernel;
 }
 void batq_debug_force_quantizer(int32_t which) { g_force_quantizer.store(which, std::memory_order_relaxed); }
 void batq_debug_force_gemm_kernel(int32_t which) { g_force_gemm_kernel.store(which, std::memory_order_relaxed); }
