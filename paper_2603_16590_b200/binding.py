@@ -117,7 +117,7 @@ def _load_call_shim(lib):
     loader = importlib.machinery.ExtensionFileLoader("_pycall", path)
     _CALL = importlib.util.module_from_spec(importlib.util.spec_from_loader("_pycall", loader))
     loader.exec_module(_CALL)
-    _CALL.setup(torch.float32)
+    _CALL.setup(torch.float32, torch.Tensor)
     for name in ("batq_linear_w4a4", "batq_linear_w4a8", "batq_quantize_act", "batq_quantize_act_mxfp8"):
         _ADDRESS[name] = C.cast(getattr(lib, name), _P).value
 

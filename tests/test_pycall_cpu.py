@@ -1,6 +1,7 @@
 """The binding's CPython shim: what it hands to a C entry point (a callback stands in for it; no device)."""
 import ctypes as C
 
+import numpy as np
 import pytest
 import torch
 
@@ -42,3 +43,28 @@ def test_quantise_arguments_and_errors(call):
     with pytest.raises(TypeError):
         call.linear(addr, 0, 0)
     assert len(seen) == 1
+
+
+def test_addresses_of_any_integer_type(call, monkeypatch):
+    """An address is what int() takes (a numpy integer, as numpy's own pointers come), through the shim as through
+    ctypes; x may be anything with shape, stride() and an address; a layout is a Python int."""
+    seen = []
+    fn = C.CFUNCTYPE(C.c_int, P, P, I64, I64, I64, P, P, I32, P)(lambda *a: seen.append(a) or 0)
+    monkeypatch.setattr(binding, "_ADDRESS", {"batq_quantize_act": C.cast(fn, P).value})
+    monkeypatch.setattr(binding, "_stream", lambda: 7)
+    x = torch.empty((4, 64), dtype=torch.bfloat16)
+
+    class Rows:
+        shape = (4, 64)
+        stride = staticmethod(lambda d: 96)
+        __int__ = lambda self: 4096
+
+    top = np.uint64((1 << 64) - 256)
+    binding.batq_quantize_act(None, x, np.int64(1 << 40), top, binding.SF_MMA)
+    binding.batq_quantize_act(None, Rows(), 512, -256, binding.SF_ROWMAJOR)
+    assert seen == [(None, x.data_ptr(), 4, 64, 64, 1 << 40, int(top), 1, 7), (None, 4096, 4, 64, 96, 512, int(top), 0, 7)]
+    with pytest.raises(TypeError):
+        binding.batq_quantize_act(None, x, 256, 256, np.int32(1))
+    with pytest.raises(TypeError):
+        binding.batq_quantize_act(None, x, object(), 256, binding.SF_MMA)
+    assert len(seen) == 2
