@@ -11,6 +11,7 @@ import ctypes as C
 import importlib.machinery
 import importlib.util
 import os
+import sysconfig
 
 import numpy as np
 import torch
@@ -95,7 +96,7 @@ def lib_path() -> str:
 
 def load():
     """Loads libbatq.so (built in-tree by build.py); raises if it is missing."""
-    global _LIB
+    global _LIB, _CALL
     if _LIB is None:
         path = lib_path()
         if not os.path.exists(path):
@@ -104,22 +105,27 @@ def load():
         for name, (res, args) in SIGNATURES.items():
             fn = getattr(lib, name)
             fn.restype, fn.argtypes = res, args
-        _load_call_shim(lib)
-        _LIB = lib
+        for name in ("batq_linear_w4a4", "batq_linear_w4a8", "batq_quantize_act", "batq_quantize_act_mxfp8"):
+            _ADDRESS[name] = C.cast(getattr(lib, name), _P).value
+        _CALL = _load_call_shim()
+        _LIB = lib   # last: another thread may be in a call
     return _LIB
 
 
-def _load_call_shim(lib):
-    global _CALL
-    path = os.path.join(os.path.dirname(os.path.abspath(__file__)), "_pycall.so")
+def shim_path() -> str:
+    return os.path.join(os.path.dirname(os.path.abspath(__file__)), "_pycall" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
+
+
+def _load_call_shim():
+    """csrc/pycall.c as built for this interpreter; None where it has not been: the same calls then go through ctypes."""
+    path = shim_path()
     if not os.path.exists(path):
-        raise FileNotFoundError(f"{path} not found: run `python -m paper_2603_16590_b200.build`")
+        return None
     loader = importlib.machinery.ExtensionFileLoader("_pycall", path)
-    _CALL = importlib.util.module_from_spec(importlib.util.spec_from_loader("_pycall", loader))
-    loader.exec_module(_CALL)
-    _CALL.setup(torch.float32, torch.Tensor)
-    for name in ("batq_linear_w4a4", "batq_linear_w4a8", "batq_quantize_act", "batq_quantize_act_mxfp8"):
-        _ADDRESS[name] = C.cast(getattr(lib, name), _P).value
+    shim = importlib.util.module_from_spec(importlib.util.spec_from_loader("_pycall", loader))
+    loader.exec_module(shim)
+    shim.setup(torch.float32, torch.Tensor)
+    return shim
 
 
 def _check(status: int, where: str):
@@ -148,7 +154,7 @@ def _handle(h):   # of a Transform or Weight; NULL for none, or one that has bee
 def _quantise(name, t, x, codes, scales, scale_layout, ld, s, n):
     if _LIB is None:
         load()
-    if ld is None and s is None and n is None:
+    if _CALL is not None and ld is None and s is None and n is None:
         return _CALL.quantise(_ADDRESS[name], _handle(t), x, codes, scales, scale_layout, _stream())
     s = x.shape[0] if s is None else s
     n = x.shape[1] if n is None else n
@@ -159,7 +165,11 @@ def _quantise(name, t, x, codes, scales, scale_layout, ld, s, n):
 def _linear(name, t, w, x, y, workspace):
     if _LIB is None:
         load()
-    return _CALL.linear(_ADDRESS[name], _handle(t), _handle(w), x, y, workspace, _stream())
+    if _CALL is not None:
+        return _CALL.linear(_ADDRESS[name], _handle(t), _handle(w), x, y, workspace, _stream())
+    dt = F32 if y.dtype == torch.float32 else BF16
+    return getattr(_LIB, name)(t.handle if t else None, w.handle if w else None, _ptr(x), x.shape[0], x.stride(0), _ptr(y), dt,
+                               y.stride(0), _ptr(workspace), workspace.numel(), _stream())
 
 
 def _f32(a):

@@ -9,7 +9,8 @@ import sysconfig
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 LIB = os.path.join(HERE, "libbatq.so")
-CALL_LIB = os.path.join(HERE, "_pycall.so")   # CPython shim of the binding's calls
+# CPython shim of the binding's calls, one for each interpreter that has used this tree
+CALL_LIB = os.path.join(HERE, "_pycall" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
 CALL_SOURCE = os.path.join(HERE, "csrc", "pycall.c")
 SOURCES = [os.path.join(HERE, "csrc", "batq.cu")]
 DEPS = [os.path.join(HERE, "csrc", f) for f in os.listdir(os.path.join(HERE, "csrc"))] + [
@@ -24,13 +25,16 @@ def nvcc_command(extra=()):
 
 
 def _build_call_shim(force: bool):
+    """Without the Python headers or a C compiler there is no shim: the binding then makes its calls through ctypes."""
     if not force and os.path.exists(CALL_LIB) and os.path.getmtime(CALL_SOURCE) <= os.path.getmtime(CALL_LIB):
         return
-    res = subprocess.run(["gcc", "-O2", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], "-o", CALL_LIB, CALL_SOURCE],
-                         capture_output=True, text=True)
-    if res.returncode != 0:
-        sys.stderr.write(res.stderr)
-        raise RuntimeError("gcc failed building _pycall.so")
+    cmd = [os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], "-o", CALL_LIB, CALL_SOURCE]
+    try:
+        subprocess.run(cmd, capture_output=True, text=True, check=True)
+    except (OSError, subprocess.CalledProcessError) as e:
+        if os.path.exists(CALL_LIB):
+            os.remove(CALL_LIB)   # of an older source
+        sys.stderr.write(f"{getattr(e, 'stderr', None) or e}\n{CALL_LIB} not built: calls go through ctypes, some 2 us slower\n")
 
 
 def build(force: bool = False, verbose: bool = False) -> str:

@@ -1,5 +1,7 @@
 """The binding's CPython shim: what it hands to a C entry point (a callback stands in for it; no device)."""
 import ctypes as C
+import os
+import sysconfig
 
 import numpy as np
 import pytest
@@ -68,3 +70,44 @@ def test_addresses_of_any_integer_type(call, monkeypatch):
     with pytest.raises(TypeError):
         binding.batq_quantize_act(None, x, object(), 256, binding.SF_MMA)
     assert len(seen) == 2
+
+
+def test_without_the_shim(call, monkeypatch):
+    """Where the shim has not been built, load() works and the same arguments go through ctypes."""
+    monkeypatch.setattr(binding, "shim_path", lambda: __file__ + ".none")
+    monkeypatch.setattr(binding, "_LIB", None)
+    monkeypatch.setattr(binding, "_CALL", binding._CALL)
+    binding.load()
+    assert binding._CALL is None
+    seen = []
+    linear = C.CFUNCTYPE(C.c_int, P, P, P, I64, I64, P, I32, I64, P, SZ, P)(lambda *a: seen.append(a) or 0)
+    quantise = C.CFUNCTYPE(C.c_int, P, P, I64, I64, I64, P, P, I32, P)(lambda *a: seen.append(a) or 5)
+
+    class Fake:
+        batq_linear_w4a8, batq_quantize_act = linear, quantise
+
+    monkeypatch.setattr(binding, "_LIB", Fake)
+    monkeypatch.setattr(binding, "_stream", lambda: 7)
+    x = torch.empty((9, 96), dtype=torch.bfloat16)[1:4, :64]
+    y, ws = torch.empty((3, 40)), torch.empty(2048, dtype=torch.uint8)
+
+    class Handle:
+        handle = P(1 << 40)
+
+    binding.batq_linear_w4a8(None, Handle(), x, y, ws)
+    with pytest.raises(binding.BatqError):
+        binding.batq_quantize_act(Handle(), x, ws, np.int64(512), binding.SF_MMA)
+    assert seen == [(None, 1 << 40, x.data_ptr(), 3, 96, y.data_ptr(), binding.F32, 40, ws.data_ptr(), 2048, 7),
+                    (1 << 40, x.data_ptr(), 3, 64, 96, ws.data_ptr(), 512, 1, 7)]
+
+
+def test_shim_is_built_for_each_interpreter():
+    assert binding.shim_path() == build.CALL_LIB and sysconfig.get_config_var("EXT_SUFFIX") in build.CALL_LIB
+
+
+def test_build_without_python_headers(tmp_path, monkeypatch, capsys):
+    """No shim, a line on stderr, and the library as it was."""
+    monkeypatch.setattr(build, "CALL_LIB", str(tmp_path / "_pycall.so"))
+    monkeypatch.setenv("CC", str(tmp_path / "no-compiler"))
+    assert os.path.exists(build.build())
+    assert "ctypes" in capsys.readouterr().err and not os.path.exists(build.CALL_LIB)
