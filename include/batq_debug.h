@@ -66,6 +66,13 @@ void batq_debug_force_gemm_kernel(int32_t which);
  * forced. */
 void batq_debug_force_quantizer(int32_t which);
 
+/* Host only, no GPU needed: which units (128-token row tile, strip of 128 channels) the CTAs of the tensor-core quantiser
+ * work through on a device with sm_count SMs.  cta < 0: returns the number of CTAs launched.  Otherwise returns the
+ * number of units of CTA `cta`, in order, and writes the first max_units of them to units (host, 2 ints each:
+ * strip, row tile).  -1 for arguments out of range. */
+int32_t batq_debug_quantize_walk(int32_t n_strips, int32_t n_row_tiles, int32_t sm_count, int32_t cta, int32_t* units,
+                                 int32_t max_units);
+
 /* Number of K splits of the small-s GEMM (clamped to the number of 256-element K steps and to
  * 32, with MXFP8 activations to 8); 0 restores the automatic choice.  Scratch sizes follow it, and up to
  * 128 tokens layers for which that GEMM is considered take it. */

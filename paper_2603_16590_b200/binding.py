@@ -60,6 +60,7 @@ SIGNATURES = {
     "batq_linear_kernel_launches": (C.c_int32, [_P, _P, _I64]),
     "batq_debug_pair_schedule": (C.c_int32, [_I64, _I64, _I64, _I32, _I32, _P, _I32]),
     "batq_debug_wide_schedule": (C.c_int32, [_I64, _I64, _I64, _I32, _I32, _P, _I32]),
+    "batq_debug_quantize_walk": (C.c_int32, [_I32, _I32, _I32, _I32, _P, _I32]),
     "batq_debug_gemm_choice": (C.c_int32, [_I64, _I64, _I64, _I32, _I32, C.POINTER(_I32)]),
     "batq_linear_w4a4": (C.c_int, [_P, _P, _P, _I64, _I64, _P, _I32, _I64, _P, _SZ, _P]),
     "batq_linear_w4a4_host": (C.c_int, [_P, _P, _P, _I64, _P, _I32, _P, _P, _P, _SZ, _P]),
@@ -376,6 +377,20 @@ def batq_debug_pair_schedule(s, m, n, sm_count=148):
 def batq_debug_wide_schedule(s, m, n, sm_count=148):
     """The same for the wide-tile CTA-pair GEMM (host only)."""
     return _schedule(load().batq_debug_wide_schedule, s, m, n, sm_count)
+
+
+def batq_debug_quantize_walk(n_strips, n_row_tiles, sm_count=148):
+    """[[(strip, row tile), ...] per CTA] of the tensor-core quantiser (host only)."""
+    fn, out = load().batq_debug_quantize_walk, []
+    ctas = fn(n_strips, n_row_tiles, sm_count, -1, None, 0)
+    if ctas < 0:
+        raise ValueError("bad shape")
+    for c in range(ctas):
+        cnt = fn(n_strips, n_row_tiles, sm_count, c, None, 0)
+        buf = (_I32 * (2 * max(cnt, 1)))()
+        fn(n_strips, n_row_tiles, sm_count, c, buf, cnt)
+        out.append([(buf[2 * i], buf[2 * i + 1]) for i in range(cnt)])
+    return out
 
 
 def batq_debug_gemm_choice(s, m, n, mxfp8=False, sm_count=148):

@@ -2279,6 +2279,20 @@ int32_t batq_debug_wide_schedule(int64_t s, int64_t m, int64_t n, int32_t sm_cou
   }
   return cnt;
 }
+int32_t batq_debug_quantize_walk(int32_t n_strips, int32_t n_row_tiles, int32_t sm_count, int32_t cta, int32_t* units,
+                                 int32_t max_units) {
+  if (n_strips <= 0 || n_row_tiles <= 0 || sm_count <= 0) return -1;
+  const int grid = static_cast<int>(std::min<int64_t>(sm_count, static_cast<int64_t>(n_strips) * n_row_tiles));
+  if (cta < 0) return grid;
+  if (cta >= grid) return 0;
+  const QtWalk walk = qt_walk(qt_plan(n_strips, n_row_tiles, grid), n_row_tiles, cta);
+  QtUnit at(walk, 0);
+  for (int i = 0; i < walk.n && i < max_units && units != nullptr; ++i, at.advance(walk, 1)) {
+    units[2 * i] = at.strip;
+    units[2 * i + 1] = at.row_tile(walk);
+  }
+  return walk.n;
+}
 int32_t batq_debug_gemm_choice(int64_t s, int64_t m, int64_t n, int32_t sm_count, int32_t mxfp8, int32_t* width) {
   const bool a8 = mxfp8 != 0;
   if (s <= 0 || m <= 0 || n <= 0 || n % (a8 ? 128 : 32) != 0 || sm_count < 2) return -1;

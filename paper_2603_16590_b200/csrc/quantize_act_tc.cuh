@@ -82,11 +82,11 @@ inline QtPlan qt_plan(int n_strips, int n_row_tiles, int grid) {
   p.per = p.n_groups / p.strip_groups;
   const int rest = p.n_groups - p.per * p.strip_groups;
   const int64_t units = static_cast<int64_t>(p.strip_groups) * n_row_tiles;   // of a group of CTAs
-  // Rows [0, split) are walked in step, the rest is what the CTAs left over can do meanwhile.
-  p.split = n_row_tiles;
-  int64_t longest = p.per != 0 ? (n_row_tiles + p.per - 1) / p.per : 0;
+  // Rows [0, split) are walked in step, the rest is what the CTAs left over can do meanwhile; one of the two counts of
+  // steps gives nobody more than an even share.  No step at all where there are more groups of strips than of CTAs.
+  p.split = p.per != 0 ? n_row_tiles : 0;
   if (p.per != 0 && rest != 0) {
-    longest = INT64_MAX;
+    int64_t longest = INT64_MAX;
     const int64_t steps = units / p.n_groups;
     for (int64_t c = steps; c <= steps + 1; ++c) {
       const int64_t r = c * p.per < n_row_tiles ? c * p.per : n_row_tiles;
@@ -94,12 +94,8 @@ inline QtPlan qt_plan(int n_strips, int n_row_tiles, int grid) {
       if ((others > l ? others : l) < longest) { longest = others > l ? others : l; p.split = static_cast<int32_t>(r); }
     }
   }
-  // Ranges: fewer groups of CTAs than of strips, or an uneven split (the last wave counts for more there).
-  const int64_t even = (units + p.n_groups - 1) / p.n_groups;
-  const bool ranges = p.per == 0 || longest * 50 > even * 51;
-  if (ranges) { p.per = 0; p.split = 0; }
   const int64_t left = static_cast<int64_t>(p.strip_groups) * (n_row_tiles - p.split);
-  const int owners = ranges ? p.n_groups : rest > 0 ? rest : 1;
+  const int owners = p.per == 0 ? p.n_groups : rest > 0 ? rest : 1;
   p.units = static_cast<int32_t>(left / owners);
   p.extra = static_cast<int32_t>(left % owners);
   return p;
@@ -129,15 +125,15 @@ __host__ __device__ inline QtWalk qt_walk(const QtPlan& p, int n_row_tiles, int 
 // The walk's position, moved on without a division (every role of the CTA keeps one).
 struct QtUnit {
   int strip, row;
-  __device__ __forceinline__ QtUnit(const QtWalk& w, int skip) : strip(w.strip0), row(w.u0) {
+  __host__ __device__ __forceinline__ QtUnit(const QtWalk& w, int skip) : strip(w.strip0), row(w.u0) {
     if (row >= w.height) { const int s = row / w.height; strip += s * w.group; row -= s * w.height; }
     advance(w, skip);
   }
-  __device__ __forceinline__ void advance(const QtWalk& w, int units) {
+  __host__ __device__ __forceinline__ void advance(const QtWalk& w, int units) {
     row += units * w.us;
     while (row >= w.height) { row -= w.height; strip += w.group; }
   }
-  __device__ __forceinline__ int row_tile(const QtWalk& w) const { return w.row0 + row; }
+  __host__ __device__ __forceinline__ int row_tile(const QtWalk& w) const { return w.row0 + row; }
 };
 
 struct QuantTcParams {

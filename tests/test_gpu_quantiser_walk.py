@@ -9,10 +9,12 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("S,N", [(128 * 299 + 1, 128),       # one strip of 4 blocks: every CTA walks it
                                  (128 * 23 + 5, 5 * 128),    # single strips, every unit a CTA of its own
-                                 (128 * 120 + 5, 5 * 128),   # walked in step, three CTAs left over on the last rows
+                                 (128 * 120 + 5, 5 * 128),   # walked in step, three CTAs without units
+                                 (128 * 20 - 3, 41 * 128),   # walked in step, 25 CTAs on the last two rows
                                  (128 * 70, 6 * 128 - 32),   # pairs of strips, the last one part-filled
+                                 (128 * 50, 26 * 128),       # pairs, eight CTAs on the last five rows
                                  (128 * 37 + 1, 64 * 128),   # groups of four
-                                 (128 * 3, 145 * 128),       # walkers would leave three CTAs a third of the work: ranges
+                                 (128 * 3, 145 * 128),       # three units for all CTAs but three
                                  (128 * 3 - 7, 200 * 128),   # more strips than CTAs
                                  (257, 149 * 128 + 32)])
 @pytest.mark.parametrize("fp8", [False, True], ids=["mxfp4", "mxfp8"])
