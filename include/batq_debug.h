@@ -45,14 +45,15 @@ int32_t batq_debug_wide_schedule(int64_t s, int64_t m, int64_t n, int32_t sm_cou
  * (may be NULL) receives the width of its first column of tiles in features.  -1 for arguments out of range. */
 int32_t batq_debug_gemm_choice(int64_t s, int64_t m, int64_t n, int32_t sm_count, int32_t mxfp8, int32_t* width);
 
-/* Which prefill GEMM kernel later calls use.  0 = automatic (up to 128 tokens, and where the device
- * has an SM for every tile at once or an odd number of row tiles fills its waves, one CTA per
- * 128-token tile; else CTA pairs sharing a 256-token tile, with tiles of up to 256 features and two
- * accumulators, or tiles of up to 448 features and one, whichever the cost model expects to finish
- * first; batq_gemm_mxfp8_mxfp4 takes the swapped-operand kernel up to 48 tokens, and up to 128
- * where its K splits pay), 1 = always one CTA per tile, 2 = always CTA pairs with two accumulators,
- * 3 = always CTA pairs with wide tiles (batq_debug_force_tile_width then takes any multiple of 64
- * up to 448 and makes every column that wide). */
+/* Which prefill GEMM kernel later calls use.  0 = automatic (up to 128 tokens one CTA per 128-token tile; above, the
+ * same where the device has an SM for every 128-wide tile at once, where three row tiles of 256-wide ones nearly fill their
+ * waves, and with MXFP4 activations also on short K and where wider tiles make one to three nearly full waves -- one_cta_width
+ * in csrc/batq.cu has the rule --; else CTA pairs sharing a 256-token tile, with tiles of up to 256 features and two
+ * accumulators, or tiles of up to 448 features and one, whichever a model of their time expects to finish first;
+ * batq_gemm_mxfp8_mxfp4 takes the swapped-operand kernel up to 48 tokens, and up to 128 where its K splits
+ * pay), 1 = always one CTA per tile, 2 = always CTA pairs with two accumulators, 3 = always CTA pairs with
+ * wide tiles (batq_debug_force_tile_width then takes any multiple of 64 up to 448 and makes every column that
+ * wide).  batq_debug_gemm_choice shows which one a call takes. */
 void batq_debug_force_gemm_kernel(int32_t which);
 
 /* Which activation quantiser later calls use.  0 = automatic (up to 128 tokens the per-block ALU

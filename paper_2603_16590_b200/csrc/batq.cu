@@ -656,8 +656,10 @@ int pick_bn(int64_t s, int64_t m, int64_t n, int sm_count) {
 //   K up to 6144, one wave of 192- or most of one of 256-wide tiles, or two or three nearly full of 192-wide ones on K up
 //     to 3072: 4096 -> 6144 14.8 / 13.9 at 512, 5120 -> 7168 20.4 / 17.7 at 600, 3584 -> 4608 16.0 / 15.4 at 900, 2560 -> 10240 16.4 / 15.4 at 600,
 //     but 14336 -> 4096 29.3 / 30.7 at 640, 5120 -> 7168 17.1 / 17.2 at 450 (112 tiles): pairs move fewer bytes per K-step;
-//   three row tiles and full waves of 256-wide ones: 3584 -> 37888 35.1 / 31.9 at 333 (53.6 / 47.2), 5120 -> 37888 43.6 / 40.0
-//     (71.3 / 62.0); waves less than full: 4096 -> 28672 29.7 / 32.1 at 257; five row tiles: 60.4 / 60.5.
+//   three row tiles and full waves of 256-wide ones (a quarter of a pair's 512 rows would be padding): 12 layers of one to
+//     four such waves, 1280 to 6144 channels, at 257, 300 and 384 tokens, 0.83 to 0.94 of the pairs' time, with MXFP8 0.81 to
+//     0.96 (at 257 tokens 2048 -> 25088 18.8 / 17.2 and 25.5 / 22.7, 2560 -> 37632 28.0 / 25.2 and 39.3 / 35.5, 4096 -> 50176
+//     45.6 / 42.4 and 75.4 / 66.4); waves less than full: 4096 -> 28672 29.7 / 32.1 at 257; five row tiles: 60.4 / 60.5.
 // On 17 widths x 14 token counts (129 to 3000) 0.958 of the pairs' time with MXFP4, never above it; the best of all
 // widths 0.954.  MXFP8 0.972 and 0.965.
 int one_cta_width(int64_t s, int64_t m, int64_t n, int sm_count, bool a8) {

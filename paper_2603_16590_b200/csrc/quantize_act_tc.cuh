@@ -9,8 +9,7 @@
 // A goes from where TMA lands it in shared memory into tensor memory once (tcgen05.cp) and the six MMAs of a
 // block read it there: an MMA this narrow (32 columns, 17 cycles of arithmetic) takes as long as its operands
 // take to be fetched from shared memory, some 85 cycles for 5 KiB, and 24 of them were what a unit waited for
-// (with one term instead of three 32768 x 8192 ran at the time of its DRAM traffic).  32768 x 8192 124.5 -> 117 us,
-// 32768 x 4096 63 -> 58, with MXFP8 codes 70 -> 65.5, 2048 x 14336 16.8 -> 16.1; the same codes bit for bit.
+// (with one term instead of three 32768 x 8192 ran at the time of its DRAM traffic).  Figures: at QtPlan.
 // The accumulator row of a token is then read by one thread, which clips (Eq. 3-4),
 // derives the shared scale, rounds to E2M1 and stores 16 code bytes + 1 scale byte.
 //
@@ -60,8 +59,10 @@ static_assert(kQtDBufs * kQtGroups * 32 + kQtABufs * kQtACols <= kQtTmemCols, "t
 // (a linear copy kernel: 6.5).  So CTAs go down the rows in step: `per` groups of CTAs for every `group`
 // neighbouring strips, group number q on row tiles q, q + per, ...: whole rows of X at any time.  The CTAs
 // left over (148 of them do not divide by the strips) share the last rows, in ranges.
-// 32768 x 8192 135 -> 111 us, 32768 x 4096 67.5 -> 60, with MXFP8 codes 71.8 -> 65.3; 8192 x 18944 (more strips
-// than CTAs: ranges over groups of strips) 76 -> 69 with groups of 4, 72 without.
+// This walk and X by way of tensor memory together, against contiguous ranges and X from shared memory, in turn on one GPU
+// (graphs of calls): 2048 x 4096 9.7 -> 8.4 us, 8192 x 3584 19.2 -> 15.8, 3000 x 13824 24.4 -> 20.6, 20000 x 5216 81 -> 54, with
+// MXFP8 codes 5000 x 7168 23.6 -> 21.0; single calls over changing buffers 32768 x 8192 149 -> 130.  The same codes bit
+// for bit.  More strips than CTAs (8192 x 18944): ranges over groups of four strips, 5 % better than of single ones.
 struct QtPlan {                  // of a launch
   int32_t group;                 // neighbouring strips that go together
   int32_t strip_groups, n_groups;
