@@ -145,7 +145,8 @@ void batq_debug_mma_peak_second_width(int32_t bn2);
 /* on != 0 (kind::mxf4, one accumulator): the MMAs are issued by the CTA-pair GEMM's own loop, statement
  * for statement (a wait on a completed barrier phase, a fence, the scale copies into alternating
  * slots, four MMAs from descriptors that depend on a run-time stage index and a commit per K-step),
- * on the same resident operands: what that loop costs with the operand stream taken away. */
+ * on the same resident operands: what that loop costs with the operand stream taken away.  Left out
+ * is the GEMM's wait for the MMAs that read a scale slot before: every copy here writes the same bytes. */
 void batq_debug_mma_peak_gemm_loop(int32_t on);
 /* Tensor-memory column at which the loops below keep their scale factors: a multiple of 4 behind
  * the accumulators (from 256, from 448 with a second accumulator) up to 488; anything else = right

@@ -611,7 +611,7 @@ batq_status make_y_tmap(CUtensorMap* map, const void* base, int64_t rows, int64_
 // Below half a wave of 128-wide tiles: twice as many 64-wide ones where K is short (a few dozen CTAs cannot pull the
 // weights fast enough, a CTA streams what its ring keeps in flight), not where the activation tile, loaded by
 // twice as many CTAs, has many K-steps.  Whole layers of 64, 100 and 128 tokens, 64- / 128-wide: 1024 -> 1024 5.1 / 5.5 us,
-// 2048 -> 2048 6.3 / 6.8, 3072 -> 3072 8.3 / 8.7, 4096 -> 1024 8.7 / 9.0 (8 tiles), but 3584 -> 4608 9.5 / 9.0, 4096 -> 4096 9.93 / 9.84, 4096 ->
+// 2048 -> 2048 6.3 / 6.8, 3072 -> 3072 8.3 / 8.7, 4096 -> 1024 8.7 / 9.0 (8 tiles), but 3584 -> 4608 9.5 / 9.0, 4096 -> 4096 9.75 / 9.4 at 75 (at 64 and 128 within 1 % of one another), 4096 ->
 // 8192 10.9 / 10.5, 5120 -> 5120 11.5 / 11.1, 8192 -> 1024 14.6 / 14.0.
 inline bool narrow_tiles_pay(int64_t tiles128, int64_t k_steps, int sm_count) {
   return tiles128 * 2 <= sm_count && (k_steps <= 12 || (k_steps <= 16 && tiles128 * 8 <= sm_count));

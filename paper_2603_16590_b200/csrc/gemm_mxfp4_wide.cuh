@@ -21,10 +21,15 @@
 //
 // with a = min(bn, 256), b = bn - a.  Work distribution, tile numbering, segments of column widths
 // and barriers are those of gemm_mxfp4_pair.cuh (PairParams, PairWalk), with widths up to 448.
-// The scale factors of a K-step go through ONE 40-column slot of tensor memory behind the
-// accumulators (8 for the activations, 2 x 16 for four 128-row atoms of weight scales):
-// tcgen05.cp and tcgen05.mma of one thread execute in issue order, so the copy for step k+1 cannot
-// overtake the MMAs of step k that still read the slot.  No load carries a multicast qualifier.
+// The scale factors go through the 64 columns of tensor memory behind the accumulators.  The MMAs that read a slot
+// have ended before the issuer copies into it again (PTX keeps copy -> MMA in issue order, not MMA -> copy).  A tile of up
+// to 256 features has two slots of a K-step (8 columns for the activations, 2 x 12 for three 128-row atoms of
+// weight scales), as in gemm_mxfp4_pair.cuh.  A wider one needs 2 x 20 for a K-step, so it has three slots of HALF a
+// K-step: the first half's was read two steps back (the stage's empty barrier), the second half's by the first half of the
+// step before, which gets a barrier of its own; half a step and more is queued meanwhile.  A tile starts with all of them
+// free: the accumulator it waited for was complete.  Whole layers in turn with one slot and no wait: 0.999 of the time
+// (9 layers at 333 to 4096 tokens, forced onto this kernel; half-step slots for narrow tiles too: 1.045).
+// No load carries a multicast qualifier.
 #pragma once
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -49,7 +54,7 @@ struct WideCfg {
   static constexpr int kStageBytes = kABytes + kBBytes + kSfaBytes + kSfbBytes;   // 49 KiB
   static constexpr int kStages = 4;
   static constexpr int kAccCols = 448;
-  static constexpr int kSfCols = 8 + 2 * 4 * kSfbAtoms;   // 40
+  static constexpr int kSfCols = 64;                      // two slots of 32 columns or three of 20
   static constexpr int kTmemCols = 512;
   static constexpr int kStagingBufBytes = 2048;             // 32 rows x 64 bytes, one per epilogue warp
   static constexpr int kStagingBytes = kWideEpiWarps * kStagingBufBytes;
@@ -71,6 +76,7 @@ gemm_mxfp4_wide_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
   __shared__ __align__(8) uint64_t acc_full_bar;             // one per CTA
   __shared__ __align__(8) uint64_t acc_empty_bar[2];         // used in the leader only: columns [0, 256) and [256, 448)
   __shared__ __align__(8) uint64_t drain_bar;
+  __shared__ __align__(8) uint64_t half_bar;                 // leader: the MMAs of the first half of a K-step
   __shared__ uint32_t tmem_base_slot;
   __shared__ int abort_flag;
 
@@ -94,6 +100,7 @@ gemm_mxfp4_wide_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
     mbar_init(smem_u32(&acc_full_bar), 1);
     for (int i = 0; i < 2; ++i) mbar_init(smem_u32(&acc_empty_bar[i]), 2 * kWideEpiWarps);  // the epilogue warps of both CTAs
     mbar_init(smem_u32(&drain_bar), 1);
+    mbar_init(smem_u32(&half_bar), 1);
     abort_flag = 0;
     mbar_fence_init();
     tma_prefetch_desc(&tmap_a);
@@ -205,6 +212,7 @@ gemm_mxfp4_wide_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
 
       int stage = 0;
       uint32_t phase = 0;
+      uint32_t halves = 0;   // first halves of K-steps committed to half_bar so far
       uint32_t n_tile = 0;
       bool ok = true;
       PairWalk w = walk0;
@@ -223,61 +231,84 @@ gemm_mxfp4_wide_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_
         ok = __all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&acc_empty_bar[0]), (n_tile & 1u) ^ 1u, &abort_flag));
         if (!ok) break;
         tc_fence_after_sync();
+        int sf_slot = 0;   // where the first half of the next K-step's scales go
         // One K-step.  FIRST (the tile's first: the accumulators start from zero, and part b's MMAs
         // wait for part b of the accumulator) and TWO (the tile has a part b) are compile-time: the
         // elected lane's instruction stream between two MMAs holds no run-time branch.
         auto k_step = [&](auto first_c, auto two_c) {
           constexpr bool FIRST = decltype(first_c)::value;
           constexpr bool TWO = decltype(two_c)::value;
-          ok = __all_sync(0xFFFFFFFFu, mbar_wait(full0 + 8u * stage, phase, &abort_flag));
+          const int back = stage >= 2 ? stage - 2 : stage + Cfg::kStages - 2;
+          ok = __all_sync(0xFFFFFFFFu, (FIRST || mbar_wait(empty0 + 8u * back, back < stage ? phase : phase ^ 1u, &abort_flag)) &&
+                                           mbar_wait(full0 + 8u * stage, phase, &abort_flag));
           if (!ok) return;
           tc_fence_after_sync();
           const uint32_t soff = static_cast<uint32_t>(stage * (Cfg::kStageBytes >> 4));
           const uint64_t adesc = ab_desc0 + soff;
           const uint64_t bdesc = adesc + (Cfg::kABytes >> 4);
           const uint64_t sfd = sf_desc0 + soff;
-          const uint32_t sfa_col = sf_tmem0;
-          const uint32_t sfb_col = sfa_col + 8 + sfb_sub;
+          constexpr int kAtoms = TWO ? Cfg::kSfbAtoms : 3;   // 256 weight rows from a multiple of 64 touch three
+          constexpr uint32_t kHalfCols = 4 + 4 * kAtoms;
+          const uint32_t col0 = sf_tmem0 + sf_slot * kHalfCols;
+          const uint32_t col1 = TWO && sf_slot == 2 ? sf_tmem0 : col0 + kHalfCols;
+          auto copy_half = [&](int c) {
+            const uint32_t col = c != 0 ? col1 : col0;
+            tc_cp_32x128b_warpx4_pair(col, sfd + 32 * c);
+#pragma unroll
+            for (int rt = 0; rt < kAtoms; ++rt)
+              tc_cp_32x128b_warpx4_pair(col + 4 + 4 * rt, sfd + ((Cfg::kSfaBytes + rt * 1024 + c * 512) >> 4));
+          };
+          auto mma = [&](int kb, bool part_b, uint32_t accumulate) {
+            const uint32_t sfid = (kb & 1) * 2, col = (kb >> 1) != 0 ? col1 : col0;
+            const uint32_t sa = col | (sfid << 30), sb = (col + 4 + sfb_sub) | (sfid << 30);
+            if (part_b)   // weight rows 256.. of the tile: eight scale columns (256 rows) further on
+              tc_mma_mxf4_pair(tmem_base + 256, adesc + 2 * kb, bdesc + b_part_b + 2 * kb, (kb & 1) ? ib1 : ib0, sa, sb + 8, accumulate);
+            else
+              tc_mma_mxf4_pair(tmem_base, adesc + 2 * kb, bdesc + 2 * kb, (kb & 1) ? ia1 : ia0, sa, sb, accumulate);
+          };
           if (elect_one()) {
-            tc_cp_32x128b_warpx4_pair(sfa_col, sfd);
-            tc_cp_32x128b_warpx4_pair(sfa_col + 4, sfd + 32);
+            copy_half(0);
+            if (!TWO || FIRST) copy_half(1);
 #pragma unroll
-            for (int rt = 0; rt < Cfg::kSfbAtoms; ++rt)
+            for (int kb = 0; kb < (TWO && !FIRST ? 2 : 4); ++kb) {
+              mma(kb, false, (FIRST && kb == 0) ? 0u : 1u);
+              if (TWO && !FIRST) mma(kb, true, 1u);
+            }
+          }
+          if (TWO && !FIRST) {
+            __syncwarp();
+            ok = __all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&half_bar), (halves & 1u) ^ 1u, &abort_flag));
+            if (!ok) return;
+            ++halves;
+            tc_fence_after_sync();
+            if (elect_one()) {
+              tc_commit_pair_local(smem_u32(&half_bar));
+              copy_half(1);
 #pragma unroll
-              for (int c = 0; c < 2; ++c)
-                tc_cp_32x128b_warpx4_pair(sfa_col + 8 + c * 4 * Cfg::kSfbAtoms + 4 * rt,
-                                          sfd + ((Cfg::kSfaBytes + rt * 1024 + c * 512) >> 4));
-#pragma unroll
-            for (int kb = 0; kb < 4; ++kb) {
-              const uint32_t c = kb >> 1;
-              const uint32_t sfid = (kb & 1) * 2;
-              const uint32_t sa = (sfa_col + 4 * c) | (sfid << 30);
-              const uint32_t sb = (sfb_col + c * 4 * Cfg::kSfbAtoms) | (sfid << 30);
-              tc_mma_mxf4_pair(tmem_base, adesc + 2 * kb, bdesc + 2 * kb, (kb & 1) ? ia1 : ia0, sa, sb,
-                               (FIRST && kb == 0) ? 0u : 1u);
-              if (TWO && !FIRST)   // weight rows 256.. of the tile: eight scale columns (256 rows) further on
-                tc_mma_mxf4_pair(tmem_base + 256, adesc + 2 * kb, bdesc + b_part_b + 2 * kb, (kb & 1) ? ib1 : ib0, sa,
-                                 sb + 8, 1u);
+              for (int kb = 2; kb < 4; ++kb) {
+                mma(kb, false, 1u);
+                mma(kb, true, 1u);
+              }
             }
           }
           if (TWO && FIRST) {   // part a's MMAs are under way, now part b
-            ok = __all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&acc_empty_bar[1]), (n_tile & 1u) ^ 1u, &abort_flag));
+            ok = __all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&acc_empty_bar[1]), (n_tile & 1u) ^ 1u, &abort_flag) &&
+                                             mbar_wait(smem_u32(&half_bar), (halves & 1u) ^ 1u, &abort_flag));
             if (!ok) return;
+            ++halves;
             tc_fence_after_sync();
             if (elect_one()) {
 #pragma unroll
               for (int kb = 0; kb < 4; ++kb) {
-                const uint32_t c = kb >> 1;
-                const uint32_t sfid = (kb & 1) * 2;
-                tc_mma_mxf4_pair(tmem_base + 256, adesc + 2 * kb, bdesc + b_part_b + 2 * kb, (kb & 1) ? ib1 : ib0,
-                                 (sfa_col + 4 * c) | (sfid << 30), (sfb_col + 8 + c * 4 * Cfg::kSfbAtoms) | (sfid << 30),
-                                 kb != 0 ? 1u : 0u);
+                mma(kb, true, kb != 0 ? 1u : 0u);
+                if (kb == 1) tc_commit_pair_local(smem_u32(&half_bar));
               }
             }
           }
           if (elect_one()) tc_commit_pair(empty0 + 8u * stage, 3);  // frees the stage in both CTAs
           __syncwarp();
           if (++stage == Cfg::kStages) { stage = 0; phase ^= 1u; }
+          sf_slot = TWO ? (sf_slot == 0 ? 2 : sf_slot - 1) : sf_slot ^ 2;
         };
         using yes = std::integral_constant<bool, true>;
         using no = std::integral_constant<bool, false>;

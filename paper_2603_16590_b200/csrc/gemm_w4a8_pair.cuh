@@ -35,7 +35,7 @@ struct A8PairCfg {
   static constexpr int kSlot1Width = 192;
   static constexpr int kAccCols = 448;
   static constexpr int kSfCols = 4 + 4 * kSfbAtoms;       // scale columns of one K-step
-  static constexpr int kSfSlots = 2;
+  static constexpr int kSfSlots = 4;
   static constexpr int kTmemCols = 512;
   static constexpr int kStagingBufs = 2;
   static constexpr int kStagingBytes = 4 * kStagingBufs * 4096;
@@ -201,7 +201,7 @@ gemm_w4a8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_c
 
       int stage = 0;
       uint32_t phase = 0;
-      uint32_t g = 0;  // K-steps issued so far: the scale slot alternates with it
+      uint32_t g = 0;  // K-steps issued so far: the scale slot goes with it
       bool ok = true;
       PairWalk w = walk0;
       PairTile t;
@@ -217,14 +217,17 @@ gemm_w4a8_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_c
         tc_fence_after_sync();
         const uint32_t d_tmem = tmem_base + acc * Cfg::kSlot1Col;
         for (int kt = 0; kt < p.k_steps; ++kt, ++g) {
-          ok = __all_sync(0xFFFFFFFFu, mbar_wait(full0 + 8u * stage, phase, &abort_flag));
+          // the MMAs four steps back, which read the scale slot that is about to be overwritten
+          const int back = stage >= Cfg::kSfSlots ? stage - Cfg::kSfSlots : stage + Cfg::kStages - Cfg::kSfSlots;
+          ok = __all_sync(0xFFFFFFFFu, mbar_wait(empty0 + 8u * back, back < stage ? phase : phase ^ 1u, &abort_flag) &&
+                                           mbar_wait(full0 + 8u * stage, phase, &abort_flag));
           if (!ok) break;
           tc_fence_after_sync();
           const uint32_t soff = static_cast<uint32_t>(stage * (Cfg::kStageBytes >> 4));
           const uint64_t adesc = ab_desc0 + soff;
           const uint64_t bdesc = adesc + (Cfg::kABytes >> 4);
           const uint64_t sfd = sf_desc0 + soff;
-          const uint32_t sfa_col = sf_tmem0 + (g & 1u) * Cfg::kSfCols;
+          const uint32_t sfa_col = sf_tmem0 + (g % Cfg::kSfSlots) * Cfg::kSfCols;
           const uint32_t sfb_col = sfa_col + 4 + sfb_sub;
           if (elect_one()) {
             tc_cp_32x128b_warpx4_pair(sfa_col, sfd);

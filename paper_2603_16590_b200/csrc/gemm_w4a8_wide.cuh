@@ -29,12 +29,13 @@ struct A8WideCfg {
   static constexpr int kStages = 4;
   static constexpr int kAccCols = 448;
   static constexpr int kSfCols = 4 + 4 * kSfbAtoms;       // 20
+  static constexpr int kSfSlots = 3;
   static constexpr int kTmemCols = 512;
   static constexpr int kStagingBufBytes = 2048;           // 32 rows x 64 bytes, one per epilogue warp
   static constexpr int kStagingBytes = kWideEpiWarps * kStagingBufBytes;
   static constexpr int kSmemBytes = kStages * kStageBytes + kStagingBytes + 1024;
   static constexpr int kBRowTxBytes = 64;                 // what the TMA unit counts per widened weight row of a K-step
-  static_assert(kAccCols + kSfCols <= kTmemCols, "tensor memory budget");
+  static_assert(kAccCols + kSfSlots * kSfCols <= kTmemCols, "tensor memory budget");
   static_assert(kSmemBytes <= 232448, "shared memory budget");
 };
 
@@ -184,6 +185,7 @@ gemm_w4a8_wide_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_c
 
       int stage = 0;
       uint32_t phase = 0;
+      int sf_slot = 0;   // scale slot of the next K-step
       uint32_t n_tile = 0;
       bool ok = true;
       PairWalk w = walk0;
@@ -206,14 +208,17 @@ gemm_w4a8_wide_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_c
         auto k_step = [&](auto first_c, auto two_c) {
           constexpr bool FIRST = decltype(first_c)::value;
           constexpr bool TWO = decltype(two_c)::value;
-          ok = __all_sync(0xFFFFFFFFu, mbar_wait(full0 + 8u * stage, phase, &abort_flag));
+          // the MMAs three steps back, which read the scale slot that is about to be overwritten
+          const int back = stage >= Cfg::kSfSlots ? stage - Cfg::kSfSlots : stage + Cfg::kStages - Cfg::kSfSlots;
+          ok = __all_sync(0xFFFFFFFFu, mbar_wait(empty0 + 8u * back, back < stage ? phase : phase ^ 1u, &abort_flag) &&
+                                           mbar_wait(full0 + 8u * stage, phase, &abort_flag));
           if (!ok) return;
           tc_fence_after_sync();
           const uint32_t soff = static_cast<uint32_t>(stage * (Cfg::kStageBytes >> 4));
           const uint64_t adesc = ab_desc0 + soff;
           const uint64_t bdesc = adesc + (Cfg::kABytes >> 4);
           const uint64_t sfd = sf_desc0 + soff;
-          const uint32_t sfa_col = sf_tmem0;
+          const uint32_t sfa_col = sf_tmem0 + sf_slot * Cfg::kSfCols;
           const uint32_t sfb_col = sfa_col + 4 + sfb_sub;
           if (elect_one()) {
             tc_cp_32x128b_warpx4_pair(sfa_col, sfd);
@@ -244,6 +249,7 @@ gemm_w4a8_wide_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_c
           if (elect_one()) tc_commit_pair(empty0 + 8u * stage, 3);  // frees the stage in both CTAs
           __syncwarp();
           if (++stage == Cfg::kStages) { stage = 0; phase ^= 1u; }
+          if (++sf_slot == Cfg::kSfSlots) sf_slot = 0;
         };
         using yes = std::integral_constant<bool, true>;
         using no = std::integral_constant<bool, false>;

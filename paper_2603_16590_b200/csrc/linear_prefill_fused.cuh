@@ -513,7 +513,10 @@ linear_prefill_fused_kernel(const __grid_constant__ CUtensorMap tmap_x, const __
         tc_fence_after_sync();
         const uint32_t d_tmem = tmem_base + acc * Cfg::kSlot1Col;
         for (int kt = 0; kt < p.k_steps; ++kt, ++g) {
-          ok = __all_sync(0xFFFFFFFFu, mbar_wait(full0 + 8u * stage, phase, &abort_flag));
+          // the MMAs two steps back, which read the scale slot that is about to be overwritten
+          const int back = stage >= Cfg::kSfSlots ? stage - Cfg::kSfSlots : stage + Cfg::kStages - Cfg::kSfSlots;
+          ok = __all_sync(0xFFFFFFFFu, mbar_wait(empty0 + 8u * back, back < stage ? phase : phase ^ 1u, &abort_flag) &&
+                                           mbar_wait(full0 + 8u * stage, phase, &abort_flag));
           if (!ok) break;
           tc_fence_after_sync();
           const uint32_t soff = static_cast<uint32_t>(stage * (Cfg::kStageBytes >> 4));
