@@ -361,6 +361,8 @@ quantize_act_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_
         ok = __all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&d_full[old % kQtDBufs]), static_cast<uint32_t>(old / kQtDBufs) & 1u, &abort_flag));
         if (!ok) break;
       }
+      const uint32_t d_bar = smem_u32(&d_empty[buf]), d_parity = (static_cast<uint32_t>(it / kQtDBufs) & 1u) ^ 1u;
+      const bool d_free = __all_sync(0xFFFFFFFFu, mbar_try_wait(d_bar, d_parity));   // mostly so, and X is what the issuer waits for
       ok = __all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&x_full[stage]), phase, &abort_flag));
       if (!ok) break;
       tc_fence_after_sync();
@@ -377,10 +379,12 @@ quantize_act_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_
           tc_cp_128x256b(a_tmem + 8 * c, a_stage + static_cast<uint32_t>(((c >> 2) * kQtBoxBytes + (c & 3) * 32) >> 4));
         tc_commit(smem_u32(&x_empty[stage]));
       }
-      __syncwarp();
-      ok = __all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&d_empty[buf]), (static_cast<uint32_t>(it / kQtDBufs) & 1u) ^ 1u, &abort_flag));
-      if (!ok) break;
-      tc_fence_after_sync();
+      if (!d_free) {
+        __syncwarp();
+        ok = __all_sync(0xFFFFFFFFu, mbar_wait(d_bar, d_parity, &abort_flag));
+        if (!ok) break;
+        tc_fence_after_sync();
+      }
       if (elect_one()) {
 #pragma unroll
         for (int g = 0; g < kQtGroups; ++g) {
